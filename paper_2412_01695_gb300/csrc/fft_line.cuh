@@ -11,12 +11,18 @@
 // transform of the paper, no normalisation); DIR = -1 computes the forward sum with
 // e^{-2 pi i n k / N} (the 1/N_r factor is applied by the caller).
 //
+// T is float, double, or long long: the 64-bit block fixed point of fixed.cuh, whose products
+// with the constants are integer multiply-adds.
+//
 // Output order: the transform is computed in place; X_k is left in register slot
 // fft_out_slot<N>(k).  Inputs are in natural order.
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
 #include <utility>
+
+#include "fixed.cuh"
 
 // host-and-device, always inlined: lets the CPU self-test exercise the same templates
 #define PWK_HD __host__ __device__ __forceinline__
@@ -65,6 +71,7 @@ __host__ __device__ constexpr double sin2pi(long e, long n) { return cos2pi(4 * 
 template <typename T> struct C2;
 template <> struct C2<double> { using type = double2; };
 template <> struct C2<float> { using type = float2; };
+template <> struct C2<long long> { using type = longlong2; };
 template <typename T> using c2_t = typename C2<T>::type;
 
 template <typename V> PWK_HD V cadd(V a, V b) { return V{a.x + b.x, a.y + b.y}; }
@@ -121,6 +128,19 @@ PWK_HD c2_t<T> twiddle(c2_t<T> v) {
     return c2_t<T>{-v.x, -v.y};
   } else if constexpr (4 * e == 3 * N) {
     return cmul_i(v, -DIR);
+  } else if constexpr (std::is_same<T, long long>::value) {
+    if constexpr (8 * e % N == 0) {   // |cos| = |sin|: one product per component
+      constexpr long long h = fx_cos2pi(1, 8);
+      constexpr bool cp = cos2pi(e, N) > 0, sp = DIR * sin2pi(e, N) > 0;
+      const T a = v.x + v.y, d = v.x - v.y;
+      if constexpr (cp && sp) return c2_t<T>{fx_mulc<h>(d), fx_mulc<h>(a)};
+      else if constexpr (cp) return c2_t<T>{fx_mulc<h>(a), fx_mulc<-h>(d)};
+      else if constexpr (sp) return c2_t<T>{fx_mulc<-h>(a), fx_mulc<h>(d)};
+      else return c2_t<T>{fx_mulc<-h>(d), fx_mulc<-h>(a)};
+    } else {
+      constexpr long long c = fx_cos2pi(e, N), s = DIR * fx_sin2pi(e, N);
+      return c2_t<T>{fx_mulc2<c, -s>(v.x, v.y), fx_mulc2<s, c>(v.x, v.y)};
+    }
   } else {
     constexpr T c = T(cos2pi(e, N));
     constexpr T s = T(DIR * sin2pi(e, N));
@@ -158,13 +178,22 @@ template <typename T, int DIR> struct Butterfly<T, 3, DIR> {
   using V = c2_t<T>;
   template <int S>
   static PWK_HD void run(V* x) {
-    constexpr T h = T(0.5);
-    constexpr T s3 = T(DIR * 0.86602540378443864676372317075293618);  // sin(2pi/3)
     V a = x[0], b = x[S], c = x[2 * S];
     V t = cadd(b, c);
-    V m = V{a.x - h * t.x, a.y - h * t.y};
     V d = csub(b, c);
-    V r = V{-s3 * d.y, s3 * d.x};  // i * s3 * (b - c)
+    V m, r;   // m = a - t / 2, r = i s3 (b - c)
+    if constexpr (std::is_same<T, long long>::value) {
+      // an odd t is halved to the even neighbour: rounding always the same way would add up over
+      // the lines of a transform
+      m = V{a.x - ((t.x + ((t.x >> 1) & 1)) >> 1), a.y - ((t.y + ((t.y >> 1) & 1)) >> 1)};
+      constexpr long long s3 = DIR * fx_sin2pi(1, 3);
+      r = V{fx_mulc<-s3>(d.y), fx_mulc<s3>(d.x)};
+    } else {
+      constexpr T h = T(0.5);
+      constexpr T s3 = T(DIR * 0.86602540378443864676372317075293618);  // sin(2pi/3)
+      m = V{a.x - h * t.x, a.y - h * t.y};
+      r = V{-s3 * d.y, s3 * d.x};
+    }
     x[0] = cadd(a, t);
     x[S] = cadd(m, r);
     x[2 * S] = csub(m, r);
@@ -175,15 +204,24 @@ template <typename T, int DIR> struct Butterfly<T, 5, DIR> {
   using V = c2_t<T>;
   template <int S>
   static PWK_HD void run(V* x) {
-    constexpr T c1 = T(cos2pi(1, 5)), c2 = T(cos2pi(2, 5));
-    constexpr T s1 = T(DIR * sin2pi(1, 5)), s2 = T(DIR * sin2pi(2, 5));
     V a = x[0], b = x[S], c = x[2 * S], d = x[3 * S], e = x[4 * S];
     V t1 = cadd(b, e), t2 = cadd(c, d), t3 = csub(b, e), t4 = csub(c, d);
-    V p1 = V{a.x + c1 * t1.x + c2 * t2.x, a.y + c1 * t1.y + c2 * t2.y};
-    V p2 = V{a.x + c2 * t1.x + c1 * t2.x, a.y + c2 * t1.y + c1 * t2.y};
-    // q1 = i (s1 t3 + s2 t4), q2 = i (s2 t3 - s1 t4)
-    V u1 = V{s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y};
-    V u2 = V{s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y};
+    V p1, p2, u1, u2;   // q1 = i (s1 t3 + s2 t4), q2 = i (s2 t3 - s1 t4)
+    if constexpr (std::is_same<T, long long>::value) {
+      constexpr long long c1 = fx_cos2pi(1, 5), c2 = fx_cos2pi(2, 5);
+      constexpr long long s1 = DIR * fx_sin2pi(1, 5), s2 = DIR * fx_sin2pi(2, 5);
+      p1 = V{a.x + fx_mulc2<c1, c2>(t1.x, t2.x), a.y + fx_mulc2<c1, c2>(t1.y, t2.y)};
+      p2 = V{a.x + fx_mulc2<c2, c1>(t1.x, t2.x), a.y + fx_mulc2<c2, c1>(t1.y, t2.y)};
+      u1 = V{fx_mulc2<s1, s2>(t3.x, t4.x), fx_mulc2<s1, s2>(t3.y, t4.y)};
+      u2 = V{fx_mulc2<s2, -s1>(t3.x, t4.x), fx_mulc2<s2, -s1>(t3.y, t4.y)};
+    } else {
+      constexpr T c1 = T(cos2pi(1, 5)), c2 = T(cos2pi(2, 5));
+      constexpr T s1 = T(DIR * sin2pi(1, 5)), s2 = T(DIR * sin2pi(2, 5));
+      p1 = V{a.x + c1 * t1.x + c2 * t2.x, a.y + c1 * t1.y + c2 * t2.y};
+      p2 = V{a.x + c2 * t1.x + c1 * t2.x, a.y + c2 * t1.y + c1 * t2.y};
+      u1 = V{s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y};
+      u2 = V{s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y};
+    }
     V q1 = V{-u1.y, u1.x}, q2 = V{-u2.y, u2.x};
     x[0] = cadd(a, cadd(t1, t2));
     x[S] = cadd(p1, q1);

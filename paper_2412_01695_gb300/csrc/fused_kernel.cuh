@@ -20,12 +20,13 @@
 // Template parameters: T arithmetic type, TI io type (complex of TI in memory), N grid
 // size, CPLXV: V is a complex128 field and the kinetic term is absent (the
 // lattice-periodic dV psi product of the DFPT right-hand side, Eq. linear_system).
-// The real V(r) is read from a transposed copy [l2][l3][l1] (one x-line contiguous); the
-// complex dv(r) keeps the caller's [l1][l2][l3] layout.
+// V(r) and dv(r) are read from transposed copies [l2][l3][l1] (one x-line contiguous).  In FP64
+// the transforms run in the 64-bit fixed point of fixed.cuh, and the fields are limb pairs.
 #pragma once
 #include <type_traits>
 
 #include "fft_line.cuh"
+#include "fixed_block.cuh"
 #include "nl_fused.cuh"
 #include "pwk_internal.h"
 
@@ -67,9 +68,13 @@ __device__ __forceinline__ int plane_of_slot(int i, int m1lo) {
 // NL: the projector terms are applied as well (nl_fused.cuh: projections after the scatter
 // from the staged C, add-back in the gather, beta(k) read through L1/L2); compiled apart.
 template <typename T, typename TI, int N, bool CPLXV, bool NL>
-__global__ void __launch_bounds__(256) fused_kernel(FusedArgs a) {
+__global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_kernel(FusedArgs a) {
   using V = c2_t<T>;
   using VI = c2_t<TI>;
+  using A = fft_arith_t<T>;
+  using VA = c2_t<A>;
+  constexpr bool FX = std::is_same<A, long long>::value;
+  static_assert(FX || !CPLXV, "the transfer form is FP64");
   extern __shared__ __align__(16) unsigned char smem_raw[];
 
   const int item = blockIdx.x;
@@ -94,23 +99,33 @@ __global__ void __launch_bounds__(256) fused_kernel(FusedArgs a) {
   const int ns = a.nstick[k];
   const int zs = a.zs, P = a.P, L = a.L;
 
-  V* Z = reinterpret_cast<V*>(smem_raw);
-  V* Y = Z + (size_t)a.nstick_max * zs;
-  V* psis = Y + (size_t)P * N * L;
-  short* sid = reinterpret_cast<short*>(psis + a.npw_in_max);
+  VA* Z = reinterpret_cast<VA*>(smem_raw);
+  VA* Y = Z + (size_t)a.nstick_max * zs;
+  // FP32: C(G) staged; fixed point: the shifts of the x lines [N][L], y lines [P][N] and sticks,
+  // and C is read from global memory (the second and third reads hit L1)
+  V* psis = reinterpret_cast<V*>(Y + (size_t)P * N * L);
+  short* sid = reinterpret_cast<short*>(psis + (FX ? 0 : a.npw_in_max));
+  unsigned char* sx = reinterpret_cast<unsigned char*>(sid + P * N);
+  unsigned char* sy = sx + N * L;
+  unsigned char* sz = sy + P * N;
 
   const VI* pin = static_cast<const VI*>(a.in) + ((size_t)k * a.nvec_in + vin) * a.npw_in_max;
   VI* pout = static_cast<VI*>(a.out) + ((size_t)k * a.nvec_out + vout) * a.npw_out_max;
 
   // ---- 0: zero the sticks, stage the stick table and C(G)
-  for (int i = tid; i < ns * zs; i += nth) Z[i] = V{T(0), T(0)};
+  for (int i = tid; i < ns * zs; i += nth) Z[i] = VA{A(0), A(0)};
   {
     const short* sk = a.sid + (size_t)k * P * N;
     for (int i = tid; i < P * N; i += nth) sid[i] = sk[i];
   }
-  for (int g = tid; g < npi; g += nth) {
-    VI v = pin[g];
-    psis[g] = V{T(v.x), T(v.y)};
+  FxScale scale{1.0, 0.0, 0, false};
+  if constexpr (FX) {
+    scale = fx_block_scale(pin, npi, fx_scratch_at(sz + a.nstick_max));   // synchronises the block
+  } else {
+    for (int g = tid; g < npi; g += nth) {
+      VI v = pin[g];
+      psis[g] = V{T(v.x), T(v.y)};
+    }
   }
   __syncthreads();
 
@@ -121,20 +136,24 @@ __global__ void __launch_bounds__(256) fused_kernel(FusedArgs a) {
     const int* gin = a.gin + (size_t)k * a.npw_in_max;
     for (int g = tid; g < npi; g += nth) {
       const int m = gin[g];
-      Z[(m >> 8) * zs + (m & 255)] = psis[g];
+      if constexpr (FX) Z[(m >> 8) * zs + (m & 255)] = fx_from(scale, pin[g]);
+      else Z[(m >> 8) * zs + (m & 255)] = psis[g];
     }
   }
   const V* nl_bk = nl ? static_cast<const V*>(a.beta) + (size_t)k * a.nkb * a.npw_beta : nullptr;
-  if (nl) nl_fused_project<T>(a, nl_bk, a.npw_beta, psis, npi, nls);
+  if constexpr (nl) {
+    if constexpr (FX) nl_fused_project<T>(a, nl_bk, a.npw_beta, pin, npi, nls);
+    else nl_fused_project<T>(a, nl_bk, a.npw_beta, psis, npi, nls);
+  }
   __syncthreads();
   if (nl) nl_fused_coef<T>(a, nls);   // read after the barriers that follow
 
   // ---- 2: inverse z transforms on the sticks
   for (int s = tid; s < ns; s += nth) {
-    V x[N];
-    V* zr = Z + s * zs;
+    VA x[N];
+    VA* zr = Z + s * zs;
     PWK_SFOR(N, j, x[j] = zr[j]);
-    LineFFT<T, N, +1>::run(x);
+    LineFFT<A, N, +1>::run(x);
     PWK_SFOR(N, j, zr[j] = x[OutSlot<N, j>::value]);
   }
   __syncthreads();
@@ -145,44 +164,40 @@ __global__ void __launch_bounds__(256) fused_kernel(FusedArgs a) {
     // 3a: inverse y transforms of the carried m1 planes (Eq. yfft)
     for (int t = tid; t < P * lc; t += nth) {
       const int p = t / lc, c = t - p * lc;
-      V x[N];
+      VA x[N];
       PWK_SFOR(N, j, {
         const int s = sid[p * N + j];
-        x[j] = s >= 0 ? Z[s * zs + l0 + c] : V{T(0), T(0)};
+        x[j] = s >= 0 ? Z[s * zs + l0 + c] : VA{A(0), A(0)};
       });
-      LineFFT<T, N, +1>::run(x);
-      V* yp = Y + (size_t)p * N * L + c;
+      LineFFT<A, N, +1>::run(x);
+      VA* yp = Y + (size_t)p * N * L + c;
       PWK_SFOR(N, l2, yp[l2 * L] = x[OutSlot<N, l2>::value]);
     }
     __syncthreads();
     // 3b: x lines: inverse x (Eq. xfft), V(r) product, forward x (Eq. fwFFT, x part)
     for (int t = tid; t < N * lc; t += nth) {
       const int l2 = t / lc, c = t - l2 * lc;
-      V x[N];
+      VA x[N];
       PWK_SFOR(N, i, {
         const int p = plane_of_slot<N>(i, a.m1lo);
-        x[i] = ((unsigned)p < (unsigned)P) ? Y[((size_t)p * N + l2) * L + c] : V{T(0), T(0)};
+        x[i] = ((unsigned)p < (unsigned)P) ? Y[((size_t)p * N + l2) * L + c] : VA{A(0), A(0)};
       });
-      LineFFT<T, N, +1>::run(x);
-      V y[N];
-      const size_t vb = (size_t)l2 * N + l0 + c;
+      LineFFT<A, N, +1>::run(x);
+      VA y[N];
+      const size_t vline = ((size_t)l2 * N + l0 + c) * N;
       if constexpr (CPLXV) {
-        const double2* dv = static_cast<const double2*>(a.V);
-        PWK_SFOR(N, l1, {
-          const double2 w = dv[(size_t)l1 * N * N + vb];
-          const V u = x[OutSlot<N, l1>::value];
-          y[l1] = V{T(u.x * w.x - u.y * w.y), T(u.x * w.y + u.y * w.x)};
-        });
+        sx[l2 * L + c] = (unsigned char)fx_dv_product<N>(x, static_cast<const int4*>(a.V) + vline, y);
+      } else if constexpr (FX) {
+        sx[l2 * L + c] = (unsigned char)fx_v_product<N>(x, static_cast<const int2*>(a.V) + vline, y);
       } else {
-        // V transposed: the x-line (l2, l3) is contiguous
-        T w[N];
-        load_vline<T, N>(static_cast<const T*>(a.V) + ((size_t)l2 * N + l0 + c) * N, w);
+        A w[N];
+        load_vline<A, N>(static_cast<const A*>(a.V) + vline, w);
         PWK_SFOR(N, l1, {
-          const V u = x[OutSlot<N, l1>::value];
-          y[l1] = V{u.x * w[l1], u.y * w[l1]};
+          const VA u = x[OutSlot<N, l1>::value];
+          y[l1] = VA{u.x * w[l1], u.y * w[l1]};
         });
       }
-      LineFFT<T, N, -1>::run(y);
+      LineFFT<A, N, -1>::run(y);
       PWK_SFOR(N, i, {
         const int p = plane_of_slot<N>(i, a.m1lo);
         if ((unsigned)p < (unsigned)P) Y[((size_t)p * N + l2) * L + c] = y[OutSlot<N, i>::value];
@@ -192,10 +207,11 @@ __global__ void __launch_bounds__(256) fused_kernel(FusedArgs a) {
     // 3c: forward y transforms, written back onto the sticks
     for (int t = tid; t < P * lc; t += nth) {
       const int p = t / lc, c = t - p * lc;
-      V x[N];
-      const V* yp = Y + (size_t)p * N * L + c;
+      VA x[N];
+      const VA* yp = Y + (size_t)p * N * L + c;
       PWK_SFOR(N, l2, x[l2] = yp[l2 * L]);
-      LineFFT<T, N, -1>::run(x);
+      if constexpr (FX) sy[p * N + l0 + c] = (unsigned char)fx_align<N>(x, sx + c, L);
+      LineFFT<A, N, -1>::run(x);
       PWK_SFOR(N, j, {
         const int s = sid[p * N + j];
         if (s >= 0) Z[s * zs + l0 + c] = x[OutSlot<N, j>::value];
@@ -205,11 +221,17 @@ __global__ void __launch_bounds__(256) fused_kernel(FusedArgs a) {
   }
 
   // ---- 4: forward z transforms on the sticks
+  if constexpr (FX) {   // the m1 plane of every stick, until its own shift replaces it
+    for (int i = tid; i < P * N; i += nth)
+      if (sid[i] >= 0) sz[sid[i]] = (unsigned char)(i / N);
+    __syncthreads();
+  }
   for (int s = tid; s < ns; s += nth) {
-    V x[N];
-    V* zr = Z + s * zs;
+    VA x[N];
+    VA* zr = Z + s * zs;
     PWK_SFOR(N, j, x[j] = zr[j]);
-    LineFFT<T, N, -1>::run(x);
+    if constexpr (FX) sz[s] = (unsigned char)fx_align<N>(x, sy + sz[s] * N, 1);
+    LineFFT<A, N, -1>::run(x);
     PWK_SFOR(N, j, zr[j] = x[OutSlot<N, j>::value]);
   }
   __syncthreads();
@@ -217,21 +239,37 @@ __global__ void __launch_bounds__(256) fused_kernel(FusedArgs a) {
   // ---- 5: gather with 1/N_r; kinetic term
   {
     const int* gout = a.gout + (size_t)k * a.npw_out_max;
-    const T sc = T(a.scale);
+    double scd = a.scale;
+    int vexp = 0;
+    if constexpr (FX) {
+      vexp = a.vexp_dev != nullptr ? *a.vexp_dev : a.vexp;
+      if (scale.bad || vexp == kFxBadField) scd = __longlong_as_double(0x7ff8000000000000LL);
+      if (vexp == kFxBadField) vexp = 0;
+    }
     const double* g2k = a.g2 != nullptr ? a.g2 + (size_t)k * a.npw_out_max : nullptr;
     const bool with_s = nl && a.sout != nullptr;
     VI* sout = with_s ? static_cast<VI*>(a.sout) + ((size_t)k * a.nvec_out + vout) * a.npw_out_max : nullptr;
     for (int g = tid; g < npo; g += nth) {
       const int m = gout[g];
-      const V z = Z[(m >> 8) * zs + (m & 255)];
-      V acc = V{z.x * sc, z.y * sc};
+      const VA z = Z[(m >> 8) * zs + (m & 255)];
+      V acc;
+      if constexpr (FX) {
+        const int e = sz[m >> 8] + vexp - scale.exp;
+        const double f = fx_factor(scd, e);
+        acc = V{fx_scaled(z.x, f, e), fx_scaled(z.y, f, e)};
+      } else {
+        acc = V{z.x * T(scd), z.y * T(scd)};
+      }
       if constexpr (!CPLXV) {
         if (g2k != nullptr) {
           const T t2 = T(g2k[g]);
-          acc.x += t2 * psis[g].x;
-          acc.y += t2 * psis[g].y;
+          V c;
+          if constexpr (FX) c = pin[g];
+          else c = psis[g];
+          acc.x += t2 * c.x;
+          acc.y += t2 * c.y;
         }
-        if (nl) {   // the in and out spheres are the same here (npi == npo)
+        if constexpr (nl) {   // the in and out spheres are the same here (npi == npo)
           V h, sv;
           nl_fused_addback<T>(a, nl_bk, a.npw_beta, g, nls, with_s && a.qm != nullptr, h, sv);
           acc.x += h.x;

@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "fft_line.cuh"
+#include "fixed_block.cuh"
 #include "fused_kernel.cuh"
 #include "nl_fused.cuh"
 #include "pwk_internal.h"
@@ -45,10 +46,18 @@ struct OutOfWin {
 // NL: the nonlocal projector terms are applied in the epilogue (nl_fused.cuh) when the plan
 //     has projectors (a.nkb > 0); the kernel without them (NL false) is compiled apart, so the
 //     projector code costs it nothing.
+// FP64 (T = double): the transforms run in the 64-bit fixed point of fixed.cuh; C is scaled
+// into it by the scatter, and the gather returns to double with the shift of its z line.  What
+// bounds it now (N = 24): about 2500 integer instructions per line at two to three warps per
+// scheduler (the line takes 168 registers), then the FP64 projector sums.  Two CTAs of 192
+// threads (168 registers) ran 1280 band-k in 0.48 ms, of 128 threads (222 registers) in 0.56.
 template <typename T, typename TI, int N, int W, int MODE, bool NL>
 __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, int vout) {
   using V = c2_t<T>;
   using VI = c2_t<TI>;
+  using A = fft_arith_t<T>;
+  using VA = c2_t<A>;
+  constexpr bool FX = std::is_same<A, long long>::value;
   using Wn = Win<N, W>;
   constexpr int NW = Wn::NW;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -57,11 +66,18 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
   const int ns = a.nstick[k];
   const int zs = a.zs, L = a.L, yps = a.yps;
 
-  V* Z = reinterpret_cast<V*>(smem_raw);               // [NW*NW][zs]
-  V* Y = Z + (size_t)NW * NW * zs;                      // [NW][yps] (N x L used per plane)
+  using U = VA;
+  U* Z = reinterpret_cast<U*>(smem_raw);               // [NW*NW][zs]
+  // fixed point: the shifts of the z lines next to the square (the gather reads them while the
+  // projector terms reuse what follows), those of the x lines [ycopies][N][L] and y lines
+  // [NW][N] at the end
+  unsigned char* sz = reinterpret_cast<unsigned char*>(Z + (size_t)NW * NW * zs);   // [NW*NW]
+  U* Y = Z + (size_t)NW * NW * zs + (FX ? window_shift_elems(NW) : 0);   // [NW][yps] (N x L used per plane)
   // plane buffers: one [NW][yps] for the CTA (MODE 0) or one per warp (MODE 1), then the rows
   const int ycopies = MODE == 1 ? (int)(blockDim.x >> 5) : 1;
   short* rows = reinterpret_cast<short*>(Y + (size_t)ycopies * NW * yps);  // [nstick_max]
+  unsigned char* sx = reinterpret_cast<unsigned char*>(rows + a.nstick_max);
+  unsigned char* sy = sx + (size_t)ycopies * N * L;
 
   const VI* pin = static_cast<const VI*>(a.in) + ((size_t)k * a.nvec_in + vin) * a.npw_in_max;
   VI* pout = static_cast<VI*>(a.out) + ((size_t)k * a.nvec_out + vout) * a.npw_out_max;
@@ -69,10 +85,14 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
   // C(G) is read from global memory by the two stages that need it (scatter, kinetic term):
   // the second read hits L1/L2, and the shared memory a staged copy would take buys occupancy.
   // ---- 0: zero the stick square, stage the stick rows
-  for (int i = tid; i < NW * NW * zs; i += nth) Z[i] = V{T(0), T(0)};
+  for (int i = tid; i < NW * NW * zs; i += nth) Z[i] = U{};
   {
     const short* rk = a.sid + (size_t)k * a.nstick_max;
     for (int i = tid; i < ns; i += nth) rows[i] = rk[i];
+  }
+  FxScale scale{1.0, 0.0, 0, false};
+  if constexpr (FX) {
+    scale = fx_block_scale(pin, np, fx_scratch_at(sy + NW * N));   // synchronises the block
   }
   __syncthreads();
 
@@ -82,150 +102,211 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     for (int g = tid; g < np; g += nth) {
       const int m = gin[g];
       const VI v = pin[g];
-      Z[(m >> 8) * zs + (m & 255)] = V{T(v.x), T(v.y)};
+      if constexpr (FX) Z[(m >> 8) * zs + (m & 255)] = fx_from(scale, v);
+      else Z[(m >> 8) * zs + (m & 255)] = VA{A(v.x), A(v.y)};
     }
   }
   __syncthreads();
 
-  // ---- 2: inverse z transforms of the real sticks (inputs only in the m3 window)
-  for (int s = tid; s < ns; s += nth) {
-    V x[N];
-    V* zr = Z + rows[s] * zs;
-    PWK_SFOR(N, j, x[j] = Wn::in(j) ? zr[j] : V{T(0), T(0)});
-    LineFFTZ<T, N, +1, OutOfWin<N, W>>::run(x);
-    PWK_SFOR(N, j, zr[j] = x[OutSlot<N, j>::value]);
-  }
-  __syncthreads();
-
-  if constexpr (MODE == 0) {
-  // ---- 3: planes l3 in chunks of L
-  for (int l0 = 0; l0 < N; l0 += L) {
-    const int lc = min(L, N - l0);
-    // 3a: inverse y transforms, inputs on the m2 window of plane p
-    for (int t = tid; t < NW * lc; t += nth) {
-      const int c = t / NW, p = t - c * NW;   // plane fastest: conflict-free (see window_strides)
-      V x[N];
-      const V* zp = Z + (size_t)p * NW * zs + l0 + c;
-      PWK_SFOR(N, j, x[j] = Wn::in(j) ? zp[Wn::idx(j) * zs] : V{T(0), T(0)});
-      LineFFTZ<T, N, +1, OutOfWin<N, W>>::run(x);
-      V* yp = Y + (size_t)p * yps + c;
-      PWK_SFOR(N, l2, yp[l2 * L] = x[OutSlot<N, l2>::value]);
+  // ---- 2-4: the line passes.  Inverse z on the real sticks; per chunk of L planes inverse y on
+  // the m2 window of plane p, the x lines (inverse, V(r) product, forward, window outputs only)
+  // and forward y, window outputs back to the stick square; forward z.  MODE 1: a warp's chunks
+  // are its own.
+  const int warp = MODE == 1 ? tid >> 5 : 0, nw = MODE == 1 ? nth >> 5 : 1;
+  const int lane0 = MODE == 1 ? tid & 31 : tid, step0 = MODE == 1 ? 32 : nth;
+  U* Yc = Y + (size_t)warp * NW * yps;        // [NW][yps]: plane p row, (l2, cc) at l2 L + cc
+  auto sync_pass = [&]() {
+    if constexpr (MODE == 1) __syncwarp();
+    else __syncthreads();
+  };
+  if constexpr (!FX) {
+    for (int s = tid; s < ns; s += nth) {
+      VA x[N];
+      VA* zr = Z + rows[s] * zs;
+      PWK_SFOR(N, j, x[j] = Wn::in(j) ? zr[j] : VA{A(0), A(0)});
+      LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
+      PWK_SFOR(N, j, zr[j] = x[OutSlot<N, j>::value]);
     }
     __syncthreads();
-    // 3b: x lines: inverse x, V(r) product, forward x (window outputs only)
-    for (int t = tid; t < N * lc; t += nth) {
-      const int l2 = t / lc, c = t - l2 * lc;
-      // V(r) of the line is requested first: its latency hides behind the inverse transform
-      T w[N];
-      load_vline<T, N>(static_cast<const T*>(a.V) + ((size_t)l2 * N + l0 + c) * N, w);
-      V x[N];
-      const V* yl = Y + (size_t)l2 * L + c;
-      PWK_SFOR(N, i, x[i] = Wn::in(i) ? yl[(size_t)Wn::idx(i) * yps] : V{T(0), T(0)});
-      LineFFTZ<T, N, +1, OutOfWin<N, W>>::run(x);
-      V y[N];
-      PWK_SFOR(N, l1, {
-        const V u = x[OutSlot<N, l1>::value];
-        y[l1] = V{u.x * w[l1], u.y * w[l1]};
-      });
-      LineFFT<T, N, -1>::run(y);
-      V* yo = Y + (size_t)l2 * L + c;
-      PWK_SFOR(N, i, {
-        if constexpr (Wn::in(i)) yo[(size_t)Wn::idx(i) * yps] = y[OutSlot<N, i>::value];
-      });
-    }
-    __syncthreads();
-    // 3c: forward y transforms, window outputs written back to the stick square
-    for (int t = tid; t < NW * lc; t += nth) {
-      const int c = t / NW, p = t - c * NW;
-      V x[N];
-      const V* yp = Y + (size_t)p * yps + c;
-      PWK_SFOR(N, l2, x[l2] = yp[l2 * L]);
-      LineFFT<T, N, -1>::run(x);
-      V* zp = Z + (size_t)p * NW * zs + l0 + c;
-      PWK_SFOR(N, j, {
-        if constexpr (Wn::in(j)) zp[Wn::idx(j) * zs] = x[OutSlot<N, j>::value];
-      });
-    }
-    __syncthreads();
-  }
-  } else {
-    // ---- 3 (MODE 1): each warp carries L planes of its own through y, x, y
-    const int warp = tid >> 5, lane = tid & 31, nw = nth >> 5;
-    V* Yw = Y + (size_t)warp * NW * yps;        // [NW][yps]: plane p row, (l2, cc) at l2 L + cc
     for (int l0 = warp * L; l0 < N; l0 += nw * L) {
       const int lc = min(L, N - l0);
-      // y inverse: lane -> (plane p, column cc), inputs on the m2 window
-      for (int t = lane; t < NW * lc; t += 32) {
-        const int c = t / NW, p = t - c * NW;
-        V x[N];
-        const V* zp = Z + (size_t)p * NW * zs + l0 + c;
-        PWK_SFOR(N, j, x[j] = Wn::in(j) ? zp[Wn::idx(j) * zs] : V{T(0), T(0)});
-        LineFFTZ<T, N, +1, OutOfWin<N, W>>::run(x);
-        V* yp = Yw + (size_t)p * yps + c;
+      for (int t = lane0; t < NW * lc; t += step0) {
+        const int c = t / NW, p = t - c * NW;   // plane fastest: conflict-free (see window_strides)
+        VA x[N];
+        const VA* zp = Z + (size_t)p * NW * zs + l0 + c;
+        PWK_SFOR(N, j, x[j] = Wn::in(j) ? zp[Wn::idx(j) * zs] : VA{A(0), A(0)});
+        LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
+        VA* yp = Yc + (size_t)p * yps + c;
         PWK_SFOR(N, l2, yp[l2 * L] = x[OutSlot<N, l2>::value]);
       }
-      __syncwarp();
-      // x lines: inverse x, V(r) product, forward x (window outputs only)
-      for (int t = lane; t < N * lc; t += 32) {
+      sync_pass();
+      for (int t = lane0; t < N * lc; t += step0) {
         const int l2 = t / lc, c = t - l2 * lc;
-        T w[N];
-        load_vline<T, N>(static_cast<const T*>(a.V) + ((size_t)l2 * N + l0 + c) * N, w);
-        V x[N];
-        const V* yl = Yw + (size_t)l2 * L + c;
-        PWK_SFOR(N, i, x[i] = Wn::in(i) ? yl[(size_t)Wn::idx(i) * yps] : V{T(0), T(0)});
-        LineFFTZ<T, N, +1, OutOfWin<N, W>>::run(x);
-        V y[N];
+        // V(r) of the line is requested first: its latency hides behind the inverse transform
+        A w[N];
+        load_vline<A, N>(static_cast<const A*>(a.V) + ((size_t)l2 * N + l0 + c) * N, w);
+        VA x[N], y[N];
+        VA* yl = Yc + (size_t)l2 * L + c;
+        PWK_SFOR(N, i, x[i] = Wn::in(i) ? yl[(size_t)Wn::idx(i) * yps] : VA{A(0), A(0)});
+        LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
         PWK_SFOR(N, l1, {
-          const V u = x[OutSlot<N, l1>::value];
-          y[l1] = V{u.x * w[l1], u.y * w[l1]};
+          const VA u = x[OutSlot<N, l1>::value];
+          y[l1] = VA{u.x * w[l1], u.y * w[l1]};
         });
-        LineFFT<T, N, -1>::run(y);
-        V* yo = Yw + (size_t)l2 * L + c;
+        LineFFT<A, N, -1>::run(y);
         PWK_SFOR(N, i, {
-          if constexpr (Wn::in(i)) yo[(size_t)Wn::idx(i) * yps] = y[OutSlot<N, i>::value];
+          if constexpr (Wn::in(i)) yl[(size_t)Wn::idx(i) * yps] = y[OutSlot<N, i>::value];
         });
       }
-      __syncwarp();
-      // y forward, window outputs back to the stick square (this warp's columns only)
-      for (int t = lane; t < NW * lc; t += 32) {
+      sync_pass();
+      for (int t = lane0; t < NW * lc; t += step0) {
         const int c = t / NW, p = t - c * NW;
-        V x[N];
-        const V* yp = Yw + (size_t)p * yps + c;
+        VA x[N];
+        const VA* yp = Yc + (size_t)p * yps + c;
         PWK_SFOR(N, l2, x[l2] = yp[l2 * L]);
-        LineFFT<T, N, -1>::run(x);
-        V* zp = Z + (size_t)p * NW * zs + l0 + c;
+        LineFFT<A, N, -1>::run(x);
+        VA* zp = Z + (size_t)p * NW * zs + l0 + c;
         PWK_SFOR(N, j, {
           if constexpr (Wn::in(j)) zp[Wn::idx(j) * zs] = x[OutSlot<N, j>::value];
         });
       }
-      __syncwarp();
+      sync_pass();
     }
     __syncthreads();
-  }
-
-  // ---- 4: forward z transforms of the real sticks (window outputs only)
-  for (int s = tid; s < ns; s += nth) {
-    V x[N];
-    V* zr = Z + rows[s] * zs;
-    PWK_SFOR(N, j, x[j] = zr[j]);
-    LineFFT<T, N, -1>::run(x);
-    PWK_SFOR(N, j, {
-      if constexpr (Wn::in(j)) zr[j] = x[OutSlot<N, j>::value];
-    });
+    for (int s = tid; s < ns; s += nth) {
+      VA x[N];
+      VA* zr = Z + rows[s] * zs;
+      PWK_SFOR(N, j, x[j] = zr[j]);
+      LineFFT<A, N, -1>::run(x);
+      PWK_SFOR(N, j, {
+        if constexpr (Wn::in(j)) zr[j] = x[OutSlot<N, j>::value];
+      });
+    }
+  } else {
+    // fixed point: one copy of the inverse and of the forward code for the z and y lines
+    // (unrolled over a line it is thousands of instructions, and the instruction cache holds
+    // few): stages -1 (inverse z), a chunk's y, x, y each, N (forward z).
+    // A window line reads its m >= 0 part from `pos` and its m < 0 part from `neg` (both at m
+    // times the stride).
+    unsigned char* sxc = sx + (size_t)warp * N * L;
+    // plane fastest over the threads of a y pass: conflict-free (see window_strides)
+    auto y_square = [&](int t, int l0) { return Z + ((size_t)(t % NW) * NW + W) * zs + l0 + t / NW; };
+    auto y_chunk = [&](int t) { return Yc + (size_t)(t % NW) * yps + t / NW; };
+    auto inverse_line = [&](const VA* pos, const VA* neg, int stride, VA* out, int ostride) {
+      VA x[N];
+      PWK_SFOR(N, j, {
+        if constexpr (!Wn::in(j)) x[j] = VA{A(0), A(0)};
+        else if constexpr (j <= W) x[j] = pos[j * stride];
+        else x[j] = neg[(j - N) * stride];
+      });
+      LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
+      PWK_SFOR(N, j, out[j * ostride] = x[OutSlot<N, j>::value]);
+    };
+    // ss: shifts of the inputs (fixed point), at ss[j sstride]; so: where the line's own goes
+    auto forward_line = [&](const VA* in, int stride, const unsigned char* ss, int sstride, unsigned char* so, VA* pos,
+                            VA* neg, int ostride) {
+      VA x[N];
+      PWK_SFOR(N, j, x[j] = in[j * stride]);
+      *so = (unsigned char)fx_align<N>(x, ss, sstride);
+      LineFFT<A, N, -1>::run(x);
+      PWK_SFOR(N, j, {
+        if constexpr (Wn::in(j)) {
+          if constexpr (j <= W) pos[j * ostride] = x[OutSlot<N, j>::value];
+          else neg[(j - N) * ostride] = x[OutSlot<N, j>::value];
+        }
+      });
+    };
+    auto x_line = [&](int t, int l0, int lc) {
+      const int l2 = t / lc, c = t - l2 * lc;
+      VA x[N], y[N];
+      U* yl = Yc + (size_t)l2 * L + c;
+      PWK_SFOR(N, i, x[i] = Wn::in(i) ? yl[(size_t)Wn::idx(i) * yps] : VA{A(0), A(0)});
+      LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
+      sxc[l2 * L + c] = (unsigned char)fx_v_product<N>(x, static_cast<const int2*>(a.V) + ((size_t)l2 * N + l0 + c) * N, y);
+      LineFFT<A, N, -1>::run(y);
+      PWK_SFOR(N, i, {
+        if constexpr (Wn::in(i)) yl[(size_t)Wn::idx(i) * yps] = y[OutSlot<N, i>::value];
+      });
+    };
+    for (int l0 = -1;;) {
+      const bool first = l0 < 0, last = l0 >= N;
+      const int lc = first || last ? 0 : min(L, N - l0);
+      if (!last) {
+        const int n = first ? ns : NW * lc, step = first ? nth : step0;
+        for (int t = first ? tid : lane0; t < n; t += step) {
+          const VA *pos, *neg;
+          VA* out;
+          if (first) {
+            out = Z + rows[t] * zs;
+            pos = out;
+            neg = out + N;
+          } else {
+            pos = neg = y_square(t, l0);
+            out = y_chunk(t);
+          }
+          inverse_line(pos, neg, first ? 1 : zs, out, first ? 1 : L);
+        }
+        if (first) {
+          __syncthreads();
+          l0 = warp * L;
+          if (l0 >= N) __syncthreads();   // a warp without chunks: the barrier before the last stage
+          continue;
+        }
+        sync_pass();
+        for (int t = lane0; t < N * lc; t += step0) x_line(t, l0, lc);
+        sync_pass();
+      }
+      const int n = last ? ns : NW * lc, step = last ? nth : step0;
+      for (int t = last ? tid : lane0; t < n; t += step) {
+        const VA* in;
+        VA *pos, *neg;
+        const unsigned char* ss;
+        unsigned char* so;
+        if (last) {
+          const int row = rows[t];
+          VA* zr = Z + row * zs;
+          in = pos = zr;
+          neg = zr + N;
+          ss = sy + row / NW * N;
+          so = sz + row;
+        } else {
+          in = y_chunk(t);
+          pos = neg = y_square(t, l0);
+          ss = sxc + t / NW;
+          so = sy + t % NW * N + l0 + t / NW;
+        }
+        forward_line(in, last ? 1 : L, ss, last ? 1 : L, so, pos, neg, last ? 1 : zs);
+      }
+      if (last) break;
+      l0 += nw * L;
+      if (l0 >= N) __syncthreads();
+      else sync_pass();
+    }
   }
   __syncthreads();
 
   // ---- 5: gather with 1/N_r; kinetic term
+  const int vexp = a.vexp == kFxBadField ? 0 : a.vexp;
+  const double scd = FX && (scale.bad || a.vexp == kFxBadField) ? __longlong_as_double(0x7ff8000000000000LL) : a.scale;
+  auto local = [&](int m) -> V {   // the local term of the basis vector at packed place m
+    const VA z = Z[(m >> 8) * zs + (m & 255)];
+    if constexpr (FX) {
+      const int e = sz[m >> 8] + vexp - scale.exp;
+      const double f = fx_factor(scd, e);
+      return V{fx_scaled(z.x, f, e), fx_scaled(z.y, f, e)};
+    } else {
+      const T sc = T(scd);
+      return V{z.x * sc, z.y * sc};
+    }
+  };
   if (!NL || a.nkb == 0) {
     const int* gout = a.gout + (size_t)k * a.npw_out_max;
-    const T sc = T(a.scale);
     const double* g2k = a.g2 + (size_t)k * a.npw_out_max;
     for (int g = tid; g < np; g += nth) {
-      const int m = gout[g];
-      const V z = Z[(m >> 8) * zs + (m & 255)];
+      const V z = local(gout[g]);
       const T t2 = T(g2k[g]);
       const VI cv = pin[g];
-      V acc = V{z.x * sc + t2 * T(cv.x), z.y * sc + t2 * T(cv.y)};
+      V acc = V{z.x + t2 * T(cv.x), z.y + t2 * T(cv.y)};
       pout[g] = VI{TI(acc.x), TI(acc.y)};
     }
     for (int g = np + tid; g < a.npw_out_max; g += nth) pout[g] = VI{TI(0), TI(0)};
@@ -234,17 +315,15 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     // stick square; once the square is read, beta(k) is staged over it, and the projections,
     // gamma (delta) and the add-back (S C) run from shared memory.
     const int* gout = a.gout + (size_t)k * a.npw_out_max;
-    const T sc = T(a.scale);
     const double* g2k = a.g2 + (size_t)k * a.npw_out_max;
     V* LOC = reinterpret_cast<V*>(smem_raw + a.loc_off);   // [npw_out_max] local + kinetic
     V* Cs = LOC + a.npw_out_max;                             // [npw_out_max] C in T
     V* nls = reinterpret_cast<V*>(smem_raw + a.nl_off);
     for (int g = tid; g < np; g += nth) {
-      const int m = gout[g];
-      const V z = Z[(m >> 8) * zs + (m & 255)];
+      const V z = local(gout[g]);
       const T t2 = T(g2k[g]);
       const VI cv = pin[g];
-      LOC[g] = V{z.x * sc + t2 * T(cv.x), z.y * sc + t2 * T(cv.y)};
+      LOC[g] = V{z.x + t2 * T(cv.x), z.y + t2 * T(cv.y)};
       Cs[g] = V{T(cv.x), T(cv.y)};
     }
     __syncthreads();
@@ -274,10 +353,15 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
   }
 }
 
+// Threads the register budget allows for: an FP64 line of N <= 27 fits the 168 registers of 384
+// threads per SM (a few words spilled at N = 24, 27), which lets two CTAs of 192 run on an SM.
+template <typename T, int N>
+constexpr int window_max_threads() { return sizeof(T) == 8 && N <= 27 ? 384 : 256; }
+
 // One CTA per work item of one plan: item = (k - k0) * nvec + band of a batched call, or the
 // (k, in_slot, out_slot) entry of a work list.
 template <typename T, typename TI, int N, int W, int MODE, bool NL>
-__global__ void __launch_bounds__(256) fused_window_kernel(FusedArgs a) {
+__global__ void __launch_bounds__(window_max_threads<T, N>()) fused_window_kernel(FusedArgs a) {
   const int item = blockIdx.x;
   if (a.d_count != nullptr && item >= *a.d_count) return;
   int k, vin, vout;
@@ -304,7 +388,7 @@ __global__ void __launch_bounds__(256) fused_window_kernel(FusedArgs a) {
 // is an empty slot; one outside the plans or the plan's k-points and slots is skipped and
 // flagged in the first plan's error word.
 template <typename T, typename TI, int N, int W, int MODE>
-__global__ void __launch_bounds__(256) fused_window_multi_kernel(FusedArgs a0) {
+__global__ void __launch_bounds__(window_max_threads<T, N>()) fused_window_multi_kernel(FusedArgs a0) {
   const int item = blockIdx.x;
   const int* it = a0.items + 4 * (size_t)item;
   const int p = it[0], k = it[1], vin = it[2], vout = it[3];

@@ -93,8 +93,10 @@ bool grid_supported(int N) {
 
 size_t fused_smem_bytes(int N, int elem_bytes, int nstick_max, int P, int L, int npw_in_max) {
   const int zs = (N % 2 == 0) ? N + 1 : N;
-  size_t elems = (size_t)nstick_max * zs + (size_t)P * N * L + npw_in_max;
-  return elems * elem_bytes + (size_t)P * N * sizeof(short) + 16;
+  const bool fx = elem_bytes == 16;   // FP64: line shifts instead of the staged C(G)
+  size_t elems = (size_t)nstick_max * zs + (size_t)P * N * L + (fx ? 0 : npw_in_max);
+  return elems * elem_bytes + (size_t)P * N * sizeof(short) +
+         (fx ? (size_t)N * L + (size_t)P * N + nstick_max : 0) + 16;
 }
 
 // The y pass maps thread t to (plane p = t % NW, column c = t / NW) and touches element
@@ -122,7 +124,8 @@ size_t window_smem_bytes(int N, int elem_bytes, int L, int nstick_max, int copie
   int zs, yps;
   window_strides(N, L, &zs, &yps);
   size_t elems = (size_t)NW * NW * zs + (size_t)copies * NW * yps;
-  return elems * elem_bytes + (size_t)nstick_max * sizeof(short) + 16;
+  const size_t shifts = elem_bytes == 16 ? (size_t)copies * N * L + (size_t)NW * N + 16 * (size_t)window_shift_elems(NW) : 0;
+  return elems * elem_bytes + (size_t)nstick_max * sizeof(short) + shifts + 16;
 }
 
 // ---------------------------------------------------------------- setup kernels
@@ -148,13 +151,41 @@ __global__ void to_f32_kernel(size_t n, const double* in, float* out) {
 }
 
 // Vt[(l2 N + l3) N + l1] = V[(l1 N + l2) N + l3]: one x-line of the grid contiguous
-template <typename T>
-__global__ void transpose_v_kernel(int N, const double* V, T* Vt) {
+__global__ void transpose_v_kernel(int N, const double* V, float* Vt) {
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const size_t n3 = (size_t)N * N * N;
   if (i >= n3) return;
   const int l1 = (int)(i % N), l3 = (int)((i / N) % N), l2 = (int)(i / ((size_t)N * N));
-  Vt[i] = (T)V[((size_t)l1 * N + l2) * N + l3];
+  Vt[i] = (float)V[((size_t)l1 * N + l2) * N + l3];
+}
+
+// Largest high word (sign removed) of n doubles; *out starts at 0
+__global__ void hmax_kernel(size_t n, const double* in, unsigned* out) {
+  unsigned h = 0;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    h = max(h, (unsigned)__double2hiint(in[i]) & 0x7fffffffu);
+  h = __reduce_max_sync(0xffffffffu, h);
+  if ((threadIdx.x & 31) == 0) atomicMax(out, h);
+}
+
+// Limb pairs (fixed.cuh) of a field on the grid, transposed like transpose_v_kernel: the pairs
+// hold component 2^(63 - *vexp), below 2^63 (1 - 2^-20) for a real field and 2^62 for a complex
+// one (its products have two terms).
+__global__ void fx_field_kernel(int N, int ncomp, const double* in, const unsigned* hmax, int2* out, int* vexp) {
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  const size_t n3 = (size_t)N * N * N;
+  const int e = (int)(*hmax >> 20);
+  const bool bad = e == 0x7ff;
+  // every |component| < 2^(e - 1022) (subnormal values included, e = 0); one bit more where its
+  // leading bits are all ones, so that the upper limb cannot round up to 2^31
+  const int E = *hmax == 0 ? 0 : e - 1022 + ((ncomp == 2 || (*hmax & 0xfffffu) == 0xfffffu) ? 1 : 0);
+  if (i == 0) *vexp = bad ? kFxBadField : E;
+  if (i >= n3) return;
+  const int l1 = (int)(i % N), l3 = (int)((i / N) % N), l2 = (int)(i / ((size_t)N * N));
+  for (int c = 0; c < ncomp; ++c) {
+    const double v = in[(((size_t)l1 * N + l2) * N + l3) * ncomp + c];
+    out[i * ncomp + c] = bad ? int2{0, 0} : fx_pair(__double2ll_rn(ldexp(v, 63 - E)));
+  }
 }
 
 // sum of n values by one CTA in a fixed order (the result is the same on every run)
@@ -172,6 +203,16 @@ __global__ void sum_kernel(size_t n, const double* in, double* out) {
 }
 
 static int blocks_for(size_t n, int t = 256) { return (int)((n + t - 1) / t); }
+
+int launch_fx_field(int N, int ncomp, const double* field, void* pairs, unsigned* hmax, int* vexp, cudaStream_t st) {
+  const size_t n3 = (size_t)N * N * N;
+  cudaError_t e = cudaMemsetAsync(hmax, 0, sizeof(unsigned), st);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(field)");
+  hmax_kernel<<<std::min(blocks_for(n3 * ncomp), 304), 256, 0, st>>>(n3 * ncomp, field, hmax); note_launch();
+  fx_field_kernel<<<blocks_for(n3), 256, 0, st>>>(N, ncomp, field, hmax, static_cast<int2*>(pairs), vexp); note_launch();
+  e = cudaGetLastError();
+  return e == cudaSuccess ? PWK_OK : cuda_fail(e, "fx_field_kernel");
+}
 
 // ---------------------------------------------------------------- sphere maps
 // Build the stick tables for input spheres (miller_in) and output spheres (miller_out).
@@ -342,7 +383,7 @@ static size_t fused_layout(const pwk_plan* p, int precision, const LaunchShape& 
     const int N = p->N, NW = 2 * (N / 4) + 1;
     int zs = 0, yps = 0;
     window_strides(N, s.L, &zs, &yps);
-    const size_t zb = r16((size_t)NW * NW * zs * V);
+    const size_t zb = r16((size_t)NW * NW * zs * V) + (V == 16 ? 16 * (size_t)window_shift_elems(NW) : 0);
     const size_t lc = r16(2 * (size_t)p->npw_max * V);
     const size_t bb = r16((size_t)p->nkb * p->npw_max * V);
     R = std::max(R, std::max(bb, zb) + lc);
@@ -583,7 +624,8 @@ FusedArgs hpsi_args(const pwk_plan* p, int precision, const void* in, void* out)
   a.L = p->shape[precision].L;
   a.zs = (p->N % 2 == 0) ? p->N + 1 : p->N;
   a.g2 = p->d_g2;
-  a.V = precision == PWK_FP64 ? static_cast<const void*>(p->d_Vt64) : static_cast<const void*>(p->d_V32);
+  a.V = precision == PWK_FP64 ? static_cast<const void*>(p->d_Vfx) : static_cast<const void*>(p->d_V32);
+  a.vexp = p->v_exp;
   a.scale = 1.0 / (double)p->Nr;
   a.err = p->d_err;
   return a;
@@ -806,8 +848,19 @@ int pwk_plan_set_launch_shape(pwk_plan* p, int precision, int kind, int threads,
   c.kind = kind;
   c.threads = threads;
   c.L = l3_chunk;
-  c.smem = kind >= 1 ? window_smem_bytes(p->N, elem, l3_chunk, p->self.nstick_max, kind == 2 ? threads / 32 : 1)
-                     : fused_smem_bytes(p->N, elem, p->self.nstick_max, p->self.P, l3_chunk, p->npw_max);
+  auto bytes = [&] {
+    return c.kind >= 1 ? window_smem_bytes(p->N, elem, c.L, p->self.nstick_max, c.kind == 2 ? threads / 32 : 1)
+                       : fused_smem_bytes(p->N, elem, p->self.nstick_max, p->self.P, c.L, p->npw_max);
+  };
+  c.smem = bytes();
+  // an FP64 window shape within a few KB of the limit (its line shifts) takes the next smaller
+  // chunk, or the CTA-wide kind: the same bits
+  const size_t slack = 2048;
+  if (precision == PWK_FP64 && kind >= 1 && c.smem > 227 * 1024 && c.smem <= 227 * 1024 + slack) {
+    if (c.L > 1) --c.L;
+    else c.kind = 1;
+    c.smem = bytes();
+  }
   if (c.smem > 227 * 1024) {
     set_error("shape needs more than 227 KB of shared memory");
     return PWK_ERR_UNSUPPORTED;
@@ -950,11 +1003,15 @@ int pwk_plan_create(pwk_plan** out, const double* A, int N1, int N2, int N3, int
     TRYC(cudaMemcpy(p->d_D32, D32.data(), sizeof(float) * nkb * nkb, cudaMemcpyHostToDevice), "cudaMemcpy(D32)");
   }
   TRY(plan_alloc(p, (void**)&p->d_V32, sizeof(float) * (size_t)p->Nr));
-  TRY(plan_alloc(p, (void**)&p->d_Vt64, sizeof(double) * (size_t)p->Nr));
-  transpose_v_kernel<float><<<blocks_for(p->Nr), 256>>>(p->N, vloc_r, p->d_V32); note_launch();
-  transpose_v_kernel<double><<<blocks_for(p->Nr), 256>>>(p->N, vloc_r, p->d_Vt64); note_launch();
+  TRY(plan_alloc(p, (void**)&p->d_Vfx, sizeof(int2) * (size_t)p->Nr));
+  transpose_v_kernel<<<blocks_for(p->Nr), 256>>>(p->N, vloc_r, p->d_V32); note_launch();
   TRYC(cudaGetLastError(), "V transpose");
-  TRYC(cudaMalloc(&d_vsum, sizeof(double)), "cudaMalloc(tmp)");
+  TRYC(cudaMalloc(&d_vsum, 2 * sizeof(double)), "cudaMalloc(tmp)");   // the sum, then the field's exponent
+  {
+    unsigned* hm = reinterpret_cast<unsigned*>(d_vsum + 1);
+    TRY(launch_fx_field(p->N, 1, vloc_r, p->d_Vfx, hm, reinterpret_cast<int*>(hm + 1), 0));
+    TRYC(cudaMemcpy(&p->v_exp, hm + 1, sizeof(int), cudaMemcpyDeviceToHost), "cudaMemcpy(vexp)");
+  }
   TRYC(cudaMemset(d_vsum, 0, sizeof(double)), "cudaMemset");
   sum_kernel<<<1, 256>>>((size_t)p->Nr, vloc_r, d_vsum); note_launch();
   TRYC(cudaGetLastError(), "sum_kernel");

@@ -96,7 +96,8 @@ struct pwk_plan {
   float* d_q32 = nullptr;
   const double* d_V = nullptr;   // caller-owned
   float* d_V32 = nullptr;         // transposed [l2][l3][l1]
-  double* d_Vt64 = nullptr;       // transposed [l2][l3][l1]
+  int2* d_Vfx = nullptr;          // transposed [l2][l3][l1], limb pairs of V 2^(63 - v_exp)
+  int v_exp = 0;
   double v_mean = 0.0;           // average of V over the grid (diagonal of the local term)
   pwk::SphereMap self;
   // window-specialised kernel tables (|m_i| <= (N-1)/4 on every sphere of the plan)
@@ -151,7 +152,10 @@ struct FusedArgs {
   int nstick_max = 0, m1lo = 0, P = 0, L = 0, zs = 0;
   int yps = 0;                     // plane stride of the y/x chunk buffer (window kernel)
   const double* g2 = nullptr;      // kinetic table [nk][npw_out_max] or null
-  const void* V = nullptr;         // real [N^3] of the arithmetic type, or complex128 dv
+  const void* V = nullptr;         // [l2][l3][l1]: float, or limb pairs (FP64), or complex limb
+                                   // pairs (transfer form)
+  int vexp = 0;                    // FP64: the field is its limb pairs times 2^(vexp - 63)
+  const int* vexp_dev = nullptr;   // the same on the device (transfer form) or null
   double scale = 1.0;              // 1/N_r
   int* err = nullptr;
   // nonlocal projector terms fused into the kernel (nl_fused.cuh); beta == null: none
@@ -169,6 +173,9 @@ struct FusedArgs {
 };
 
 size_t fused_smem_bytes(int N, int elem_bytes, int nstick_max, int P, int L, int npw_in_max);
+// limb pairs of a real (ncomp 1) or complex (ncomp 2) field [l1][l2][l3], transposed, and its
+// exponent on the device (plan.cu); enqueued on st
+int launch_fx_field(int N, int ncomp, const double* field, void* pairs, unsigned* hmax, int* vexp, cudaStream_t st);
 
 // Arguments of the nonlocal projector kernels (nonlocal.cu): phase 0 computes gamma = D lambda
 // and delta = q lambda of every item into coef; phase 1 adds sum gamma beta to out and, if
@@ -218,11 +225,14 @@ int launch_window_f32c128_nl(int N, const FusedArgs& a, int nblocks, const Launc
 // work lists over several plans of one grid (pwk_hpsi_multi), defined in hpsi_multi.cu
 int launch_window_multi_prec(int precision, int N, const FusedArgs& a, int nblocks, const LaunchShape& s,
                              cudaStream_t st);
+int launch_window_multi_f64(int N, const FusedArgs& a, int nblocks, const LaunchShape& s, cudaStream_t st);
 int launch_window_f32(int N, const FusedArgs& a, int nblocks, const LaunchShape& s, cudaStream_t st);
 int launch_window_f32c128(int N, const FusedArgs& a, int nblocks, const LaunchShape& s,
                           cudaStream_t st);
 // copies: plane buffers (1 for a CTA-wide chunk, the warp count for per-warp planes)
 size_t window_smem_bytes(int N, int elem_bytes, int L, int nstick_max, int copies);
+// 16-byte elements that hold the shifts of the (2W+1)^2 z lines (FP64 window kernel)
+__host__ __device__ constexpr int window_shift_elems(int nw) { return (nw * nw + 15) / 16; }
 // strides of the window kernel's shared buffers for chunk L (bank-conflict-free y/x passes)
 void window_strides(int N, int L, int* zs, int* yps);
 

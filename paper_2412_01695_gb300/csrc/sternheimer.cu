@@ -48,6 +48,8 @@ struct CgWork {
   int *active = nullptr, *first = nullptr, *iters = nullptr, *items = nullptr, *counters = nullptr;
   int* list = nullptr;   // pairs still iterating, compacted (cg_compact_kernel)
   int* seen = nullptr;   // iters[i] at pair i's last true residual
+  int4* dv = nullptr;    // dv(r) as limb pairs of the transfer kernel [N][N][N]
+  unsigned* dvx = nullptr;   // its largest high word, its exponent
   std::vector<void*> ptrs;
 };
 
@@ -106,6 +108,7 @@ static int ensure_cg_work(pwk_plan* p, int nocc, bool mixed) {
       (rc = calloc_(p, w, &w->first, nv)) || (rc = calloc_(p, w, &w->iters, nv)) ||
       (rc = calloc_(p, w, &w->items, nv * 3)) || (rc = calloc_(p, w, &w->list, nv)) ||
       (rc = calloc_(p, w, &w->seen, nv)) || (rc = calloc_(p, w, &w->v32, nv2)) ||
+      (rc = calloc_(p, w, &w->dv, (size_t)p->Nr)) || (rc = calloc_(p, w, &w->dvx, 2)) ||
       (rc = calloc_(p, w, &w->counters, 4))) {
     destroy_cg_work(p);
     return rc;
@@ -933,7 +936,10 @@ extern "C" int pwk_sternheimer_cg_batched(pwk_plan* pq, pwk_plan* pk, int mode, 
     a.P = pq->xfer.P;
     a.L = pq->xshape.L;
     a.zs = (pq->N % 2 == 0) ? pq->N + 1 : pq->N;
-    a.V = dv_r;
+    int* const dvexp = reinterpret_cast<int*>(w->dvx + 1);
+    if ((rc = launch_fx_field(pq->N, 2, static_cast<const double*>(dv_r), w->dv, w->dvx, dvexp, st))) return rc;
+    a.V = w->dv;
+    a.vexp_dev = dvexp;
     a.scale = 1.0 / (double)pq->Nr;
     a.err = pq->d_err;
     if ((rc = launch_fused_xfer(pq->N, a, npairs, pq->xshape, st))) return rc;

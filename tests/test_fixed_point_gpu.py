@@ -1,0 +1,143 @@
+"""FP64 H|psi> runs its transforms in 64-bit fixed point scaled per vector: vectors, fields and
+kernel kinds at which that arithmetic could go wrong, against direct Fourier sums in long double
+(the dense oracle's own FP64 sums are ten times less accurate than what is checked here).
+
+Bar: 5e-16 relative per band: FP64 roundoff of the kinetic table and the projector sums is 2e-16
+(measured with the transforms in FP64 as well), and the transforms add less, with every vector multiplied by powers of two up to 2^900 either
+way, one plane wave (the largest growth in the forward transform), components of very different
+size, zero and non-finite vectors, V constant, V = 0, V large and tiny."""
+import numpy as np
+import pytest
+
+from paper_2412_01695_gb300 import synth
+
+from gpu_util import torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+A = synth.fcc_lattice(7.5)
+B = synth.reciprocal_rows(A)
+
+
+def problem(N, V_r=None, lset=(0, 1)):
+    # the largest sphere the window kernel takes on this grid
+    ecut = ((N // 4 + 0.4) * 2 * np.pi / np.linalg.norm(A[0])) ** 2 * 0.9
+    k = synth.mp_grid(B, (1, 1, 1)) + 0.05
+    return synth.build_problem(A, np.zeros((1, 3)), lset, N, ecut, k, 4, 1, V_r=V_r, with_psi=False)
+
+
+def vectors(prob):
+    """Per k: normal components, one plane wave, components from 1 to 1e-12, zero."""
+    r = np.random.default_rng(5)
+    x = np.zeros((prob.nk, 4, prob.npw_max), complex)
+    for k in range(prob.nk):
+        n = prob.npw[k]
+        x[k, 0, :n] = r.standard_normal(n) + 1j * r.standard_normal(n)
+        x[k, 1, n // 2] = 1 - 2j
+        x[k, 2, :n] = (r.standard_normal(n) + 1j * r.standard_normal(n)) * np.logspace(0, -12, n)
+    return x
+
+
+def apply(prob, x, shape=None, path=0):
+    torch = torch_cuda()
+    from paper_2412_01695_gb300 import pwk
+    plan = pwk.plan_from_problem(prob)
+    if shape is not None:
+        plan.set_launch_shape(pwk.PWK_FP64, *shape)
+    plan.set_projector_path(path)
+    d = torch.from_numpy(x).cuda()
+    y = torch.full_like(d, complex(np.nan, np.nan))
+    pwk.hpsi_batched(plan, pwk.PWK_FP64, d, y, x.shape[1])
+    torch.cuda.synchronize()
+    plan.close()
+    return y.cpu().numpy()
+
+
+def reference(prob, k, x):
+    """H x of k-point k by direct separable sums, x [nb][npw], in long double."""
+    ld, cl = np.longdouble, np.clongdouble
+    N, n = prob.N, int(prob.npw[k])
+    pi = ld("3.14159265358979323846264338327950288")
+    i = np.arange(N)
+    E = np.exp(cl(2j) * pi * ((np.outer(i, i) % N).astype(ld)) / N)
+    m = prob.miller[k][:n] % N
+    q = prob.kpts[k][None, :] + prob.miller[k][:n] @ prob.B
+    b = prob.beta[k][:, :n].astype(cl)
+    out = []
+    for v in x[:, :n].astype(cl):
+        g = np.zeros((N, N, N), cl)
+        g[m[:, 0], m[:, 1], m[:, 2]] = v
+        for F, f in ((E, prob.V_r.astype(ld)), (E.conj(), ld(1) / N ** 3)):
+            g = np.einsum("ai,ijk->ajk", F, g)
+            g = np.einsum("bj,ajk->abk", F, g)
+            g = np.einsum("ck,abk->abc", F, g) * f
+        out.append(g[m[:, 0], m[:, 1], m[:, 2]] + np.sum(q * q, axis=1) * v + ((v @ b.conj().T) @ prob.D) @ b)
+    return np.array(out)
+
+
+def check(prob, x, y, scale=1.0):
+    for k in range(prob.nk):
+        n = prob.npw[k]
+        ref = reference(prob, k, x[k])
+        assert np.all(y[k][:, n:] == 0)
+        for b in range(x.shape[1]):
+            err = np.linalg.norm((y[k, b, :n] / scale - ref[b]).astype(complex))
+            bar = 5e-16 * max(np.linalg.norm(ref[b].astype(complex)), np.linalg.norm(x[k, b]))
+            assert err <= bar, (k, b, 5e-16 * err / max(bar, 1e-300))
+
+
+@pytest.mark.parametrize("N", [12, 15, 20, 24, 25, 27, 32])
+@pytest.mark.parametrize("kind", [0, 1, 2])
+def test_every_kind_at_every_radix(N, kind):
+    prob = problem(N)
+    x = vectors(prob)
+    check(prob, x, apply(prob, x, (kind, 128, 1 if kind == 2 else max(1, N // 8))))
+
+
+@pytest.mark.parametrize("exponent", [-1060, -900, -300, 300, 900])
+def test_vectors_of_any_magnitude(exponent):
+    prob = problem(16)
+    x = vectors(prob)
+    x[:, 2] = 0   # its range would leave the doubles
+    # 2^exponent in two exact steps; below 2^-1022 the inputs themselves lose bits
+    half = 2.0 ** (exponent // 2)
+    s = x * half * 2.0 ** (exponent - exponent // 2)
+    y = apply(prob, s)
+    if exponent == -1060:
+        assert np.all(np.isfinite(y)) and np.any(y != 0)
+        return
+    check(prob, x, y / half, 2.0 ** (exponent - exponent // 2))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("path", [2, 3])
+def test_a_non_finite_vector_spoils_only_itself(bad, path):
+    prob = problem(16)
+    x = vectors(prob)
+    x[0, 2, 5] = bad
+    y = apply(prob, x, path=path)
+    assert np.all(~np.isfinite(y[0, 2, :prob.npw[0]]))
+    y[0, 2] = 0
+    x[0, 2] = 0
+    check(prob, x, y)
+
+
+@pytest.mark.parametrize("field", ["zero", "constant", "large", "tiny", "spike", "nan"])
+def test_fields(field):
+    N = 20
+    r = np.random.default_rng(3)
+    V = {"zero": np.zeros((N,) * 3), "constant": np.full((N,) * 3, -0.75), "large": 2.0 ** 40 * r.standard_normal((N,) * 3),
+         "tiny": 2.0 ** -80 * r.standard_normal((N,) * 3), "spike": np.zeros((N,) * 3),
+         "nan": r.standard_normal((N,) * 3)}[field]
+    if field == "spike":
+        V[3, 4, 5] = -1e3
+    if field == "nan":
+        V[0, 0, 1] = np.nan
+    prob = problem(N, V_r=V, lset=(0,))
+    x = vectors(prob)
+    y = apply(prob, x)
+    if field == "nan":
+        for k in range(prob.nk):
+            assert np.all(np.isnan(y[k, :, :prob.npw[k]].real))
+        return
+    check(prob, x, y)
