@@ -3,9 +3,11 @@
 //
 // The paper runs LAPACK ZHEGV(X) converted to device routines, one thread per k, with a
 // non-recursive Cholesky (ZPOTRF2 rewritten).  Here a whole CTA works on one k:
-//   1. Cholesky S~ = L L^H (right-looking, column by column, lower triangle only);
-//   2. C = L^-1 H~ L^-H: X = L^-1 H~ by forward substitution (one thread per column), then
-//      the lower triangle of C = X L^-H by row-wise substitution (one thread per row);
+//   1. Cholesky S~ = L L^H (right-looking, column by column, lower triangle only; one warp runs
+//      a column ahead of the trailing update);
+//   2. C = L^-1 H~ L^-H: X = L^-1 H~ by blocks of rows, then the lower triangle of C = X L^-H by
+//      blocks of columns (the product with what lies before a block over all threads, then a
+//      substitution inside it);
 //   3. Householder reduction of C to a real symmetric tridiagonal T = Q^H C Q
 //      (reflectors H = I - tau v v^H, beta real, two-sided rank-2 updates of the lower
 //      triangle);
@@ -20,7 +22,13 @@
 // The kernel is bound by the FP64 pipe (1/64 of the FP32 rate on this GPU) when the batch
 // is full, so the loops count FP64 instructions: fused multiply-add chains (4 per complex
 // multiply-add), triangles visited without masked lanes, reciprocal pivots formed once,
-// reductions of the reflector step done by one warp.
+// reductions of the reflector step done by one warp.  A CTA that has an SM to itself is bound by
+// its serial parts as much: measured per phase at n = 80, 20 vectors, one CTA per SM (us, before ->
+// after the look-ahead, the blocked solves and 512 threads instead of 256): Cholesky 257 -> 208, X
+// 510 -> 307, C 514 -> 216, Householder 1516 -> 1026, eigenvalues 353 -> 265, inverse iteration
+// 200 -> 193, back-transform 411 -> 405; in all 3.80 -> 2.64 ms (FP64 pipe 45 -> 67 % busy).  n =
+// 32, 8 vectors: 0.83 -> 0.55 ms; n = 160, 40 vectors: 16.1 -> 13.4 ms; 512 problems of n = 80: 7.4
+// -> 7.5 ms.
 // A dependent vector among the first nb (pivot below 1e-6 of its diagonal) marks the k-point
 // with status PWK_ERR_NOT_POSDEF; a non-finite eigenvector, or eigenvectors of T that are not
 // orthonormal to 1e-8, mark it PWK_ERR_NUMERIC.
@@ -64,6 +72,22 @@ __device__ __forceinline__ void cfms_c(double2& s, double2 a, double2 b) {   // 
   s.y = fma(a.x, b.y, s.y);
 }
 
+// 1 / x and 1 / sqrt(x) to about an ulp: the hardware approximation (20 bits) and two Newton
+// steps.  x is normal and not near the ends of the range (pivots are clamped away from zero).
+__device__ __forceinline__ double fast_rcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(fma(-x, r, 1.0), r, r);
+  return fma(fma(-x, r, 1.0), r, r);
+}
+__device__ __forceinline__ double fast_rsqrt(double x) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double h = 0.5 * x;
+  r = fma(fma(-h * r, r, 0.5), r, r);
+  return fma(fma(-h * r, r, 0.5), r, r);
+}
+
 // Visit every (r, c) with 0 <= c <= r < m once, spread over the block: rows p and m-1-p are
 // paired (p + 1 and m - p entries, m + 1 together), so the flat index runs over
 // ceil(m/2) (m + 1) slots and the triangle masks off no lane.  Threads step their (p, o)
@@ -86,6 +110,8 @@ __device__ __forceinline__ void for_lower(int m, int tid, int nth, F f) {
   }
 }
 
+constexpr int kBlk = 16;   // rows (columns) per block of the two triangular solves
+
 // block-wide sum of a double (all threads get the result)
 __device__ double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -107,7 +133,7 @@ __device__ double2 block_sum2(double2 v, double* red) {
 // W: [nk][3][ld][ld] workspace; ev: [nk][ld][nb]; eps: [nk][nb]; status [nk]
 // nbase == nullptr: every problem has size ld.  status may be null (not written).
 // drop_out: [nk][ld] dependent-vector flags of the Cholesky step, or null.
-__global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const int* nbase,
+__global__ void __launch_bounds__(512, 2) rr_kernel(int nk, int ld, int nb, const int* nbase,
                                                  const int* active, const double2* Hr,
                                                  const double2* Sr, double2* W, double2* ev,
                                                  double* eps, int* status, unsigned char* drop_out,
@@ -122,7 +148,8 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
   if (flops != nullptr && tid == 0) atomicAdd(flops, 12.0 * n * n * n + 12.0 * n * n * nb);
   __shared__ double red[32];
   __shared__ double d[kMaxBasis], e[kMaxBasis], rc[kMaxBasis], rs[kMaxBasis];
-  __shared__ double2 tau[kMaxBasis], vv[kMaxBasis], ww[kMaxBasis];
+  __shared__ double2 tau[kMaxBasis], vv[2][kMaxBasis], ww[kMaxBasis];
+  __shared__ double hh[kMaxBasis];
   __shared__ double lam[kMaxBasis];
   __shared__ int flag;
   __shared__ unsigned char dropped[kMaxBasis];
@@ -145,72 +172,114 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
     const int r = i / n, c = i - r * n;
     if (c <= r) Lm[r * ld + c] = S[r * ld + c];
   }
-  for (int i = tid; i < n; i += nth) dropped[i] = 0;
-  __syncthreads();
-  for (int j = 0; j < n; ++j) {
+  // Warp 0 runs one column ahead: while the other warps update the rest of the trailing
+  // triangle with column j, it updates column j + 1, takes its pivot and scales it (into the
+  // other buffer of vv), so a column costs one block barrier.
+  auto pivot_column = [&](int j, int buf, const double2* src) {   // warp 0; src: column j below the diagonal
+    const double p = Lm[j * ld + j].x;
+    const bool drop = !(p > 1e-6 * S[j * ld + j].x);
+    const double ip = drop ? 1.0 : (p > 1e-280 && p < 1e280 ? fast_rsqrt(p) : 1.0 / sqrt(p));
+    __syncwarp();   // every lane has read the pivot
     if (tid == 0) {
-      const double p = Lm[j * ld + j].x;
-      const bool drop = !(p > 1e-6 * S[j * ld + j].x);
       dropped[j] = drop ? 1 : 0;
       if (drop && j < nb) flag = 1;   // the leading nb vectors must be independent
-      const double l = drop ? 1.0 : sqrt(p);
-      Lm[j * ld + j] = make_double2(l, 0.0);
-      rc[j] = 1.0 / l;
+      Lm[j * ld + j] = make_double2(drop ? 1.0 : p * ip, 0.0);
+      rc[j] = ip;
     }
-    __syncthreads();
-    const int m = n - j - 1;
-    if (dropped[j]) {
-      for (int r = j + 1 + tid; r < n; r += nth) Lm[r * ld + j] = make_double2(0.0, 0.0);
-      for (int q = tid; q < j; q += nth) Lm[j * ld + q] = make_double2(0.0, 0.0);
-      __syncthreads();
-      continue;
-    }
-    const double ipiv = rc[j];
-    for (int r = tid; r < m; r += nth) {
-      double2 v = Lm[(j + 1 + r) * ld + j];
-      v = make_double2(v.x * ipiv, v.y * ipiv);
+    for (int r = tid; r < n - j - 1; r += 32) {
+      double2 v = src[r];
+      v = drop ? make_double2(0.0, 0.0) : make_double2(v.x * ip, v.y * ip);
       Lm[(j + 1 + r) * ld + j] = v;
-      vv[r] = v;
+      vv[buf][r] = v;
     }
-    __syncthreads();
-    // trailing update of the lower triangle: L[r][c] -= L[r][j] conj(L[c][j]), c <= r
-    double2* L22 = Lm + (size_t)(j + 1) * ld + (j + 1);
-    for_lower(m, tid, nth, [&](int r, int c) { cfms_c(L22[r * ld + c], vv[r], vv[c]); });
-    __syncthreads();
+    if (drop)
+      for (int q = tid; q < j; q += 32) Lm[j * ld + q] = make_double2(0.0, 0.0);
+  };
+  __syncthreads();
+  if (tid < 32) {
+    for (int r = tid; r < n - 1; r += 32) vv[0][r] = Lm[(1 + r) * ld];
+    pivot_column(0, 0, vv[0]);
   }
+  for (int j = 0; j + 1 < n; ++j) {
+    __syncthreads();
+    const int m = n - j - 1, buf = j & 1;
+    const double2* v = vv[buf];
+    double2* L22 = Lm + (size_t)(j + 1) * ld + (j + 1);
+    const bool skip = dropped[j] != 0;
+    if (tid < 32) {
+      double2* w = vv[buf ^ 1];   // column j + 1 below its diagonal, updated
+      for (int r = tid; r < m; r += 32) {
+        double2 x = L22[r * ld];
+        if (!skip) cfms_c(x, v[r], v[0]);
+        if (r == 0) L22[0] = x;
+        else w[r - 1] = x;
+      }
+      __syncwarp();
+      pivot_column(j + 1, buf ^ 1, w);
+    } else if (!skip) {
+      // trailing update of the lower triangle: L[r][c] -= L[r][j] conj(L[c][j]), 1 <= c <= r
+      for_lower(m - 1, tid - 32, nth - 32, [&](int r, int c) {
+        cfms_c(L22[(r + 1) * ld + c + 1], v[r + 1], v[c + 1]);
+      });
+    }
+  }
+  __syncthreads();
   if (drop_out != nullptr)
     for (int i = tid; i < n; i += nth) drop_out[(size_t)k * ld + i] = dropped[i];
   if (flag) {
     if (tid == 0 && status != nullptr) status[k] = PWK_ERR_NOT_POSDEF;
     return;
   }
-  // ---- 2. X = L^-1 H (forward substitution, one column of H per thread), then the lower
-  //      triangle of C = X L^-H row by row: row r of C solves C[r][:] L^H = X[r][:], and its
-  //      entries c <= r need only the entries before them, so the lower triangle costs n^3/6
-  //      complex multiply-adds instead of the n^3/2 of a full solve.  The inverse diagonal of
-  //      L (rc) was formed once by the Cholesky step.
-  for (int c = tid; c < n; c += nth) {
-    for (int r = 0; r < n; ++r) {
+  // ---- 2. X = L^-1 H by blocks of kBlk rows (the rows above enter as one product over the whole
+  //      block, spread over every thread; then a substitution inside the block, a column per
+  //      thread), then the lower triangle of C = X L^-H by blocks of kBlk columns the same way:
+  //      row r of C solves C[r][:] L^H = X[r][:], and its entries c <= r need only the entries
+  //      before them.  The inverse diagonal of L (rc) was formed by the Cholesky step.
+  for (int r0 = 0; r0 < n; r0 += kBlk) {
+    const int nr = min(kBlk, n - r0);
+    for (int i = tid; i < nr * n; i += nth) {
+      const int r = r0 + i / n, c = i % n;
       double2 s = H[r * ld + c];
       const double2* lr = Lm + (size_t)r * ld;
-      for (int q = 0; q < r; ++q) cfms(s, lr[q], X[q * ld + c]);
-      const double il = rc[r];
-      X[r * ld + c] = make_double2(s.x * il, s.y * il);
+#pragma unroll 4
+      for (int q = 0; q < r0; ++q) cfms(s, lr[q], X[q * ld + c]);
+      X[r * ld + c] = s;
     }
+    __syncthreads();
+    for (int c = tid; c < n; c += nth)
+      for (int r = r0; r < r0 + nr; ++r) {
+        double2 s = X[r * ld + c];
+        const double2* lr = Lm + (size_t)r * ld;
+        for (int q = r0; q < r; ++q) cfms(s, lr[q], X[q * ld + c]);
+        const double il = rc[r];
+        X[r * ld + c] = make_double2(s.x * il, s.y * il);
+      }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int r = tid; r < n; r += nth) {
-    const double2* xr = X + (size_t)r * ld;
-    double2* cr = C + (size_t)r * ld;
-    for (int c = 0; c <= r; ++c) {
-      double2 s = xr[c];
-      const double2* lc = Lm + (size_t)c * ld;
-      for (int q = 0; q < c; ++q) cfms_c(s, cr[q], lc[q]);   // s -= C[r][q] conj(L[c][q])
-      const double il = rc[c];
-      cr[c] = make_double2(s.x * il, c == r ? 0.0 : s.y * il);   // C is Hermitian: real diagonal
+  for (int c0 = 0; c0 < n; c0 += kBlk) {
+    const int nc = min(kBlk, n - c0);
+    for (int i = tid; i < (n - c0) * nc; i += nth) {
+      const int r = c0 + i / nc, c = c0 + i % nc;
+      if (c > r) continue;
+      double2 s = X[r * ld + c];
+      const double2 *cr = C + (size_t)r * ld, *lc = Lm + (size_t)c * ld;
+#pragma unroll 4
+      for (int q = 0; q < c0; ++q) cfms_c(s, cr[q], lc[q]);   // s -= C[r][q] conj(L[c][q])
+      C[r * ld + c] = s;
     }
+    __syncthreads();
+    for (int r = c0 + tid; r < n; r += nth) {
+      double2* cr = C + (size_t)r * ld;
+      for (int c = c0; c <= min(r, c0 + nc - 1); ++c) {
+        double2 s = cr[c];
+        const double2* lc = Lm + (size_t)c * ld;
+        for (int q = c0; q < c; ++q) cfms_c(s, cr[q], lc[q]);
+        const double il = rc[c];
+        cr[c] = make_double2(s.x * il, c == r ? 0.0 : s.y * il);   // C is Hermitian: real diagonal
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
   // dropped vectors: decouple their row/column and park their eigenvalue above the spectrum
   // (||C||_F from the lower triangle)
   {
@@ -227,86 +296,128 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
     __syncthreads();
   }
   // ---- 3. Householder tridiagonalisation of the Hermitian C held in its lower triangle;
-  //      v_j stored in C[j+1..n-1][j] with v[0] = 1.  Per step: the reflector (warp 0), the
-  //      product w = tau C22 v (one row per thread, the upper half read through the lower
-  //      triangle), the correction w += alpha2 v (warp 0), and the rank-2 update of the lower
-  //      triangle of C22.
-  for (int j = 0; j + 1 < n; ++j) {
-    const int m = n - j - 1;       // length of x = C[j+1..n-1][j]
-    if (tid < 32) {
-      double xn2 = 0.0;
-      for (int i = 1 + tid; i < m; i += 32) {
-        const double2 v = C[(j + 1 + i) * ld + j];
-        vv[i] = v;
-        xn2 = fma(v.x, v.x, fma(v.y, v.y, xn2));
+  //      v_j stored in C[j+1..n-1][j] with v[0] = 1.  Per step: the product w = tau C22 v (P lanes
+  //      per row, the upper half read through the lower triangle), the correction
+  //      w += alpha2 v (warp 0), and the rank-2 update of the lower triangle of C22, in which
+  //      warp 0 takes the first column and goes on to the next reflector (into the other buffer
+  //      of vv) while the other warps do the rest.
+  auto reflector = [&](int j, int buf) {   // warp 0; vv[buf][0..m) holds the updated column j below its diagonal
+    const int m = n - j - 1;
+    double2* v = vv[buf];
+    double xn2 = 0.0;
+    for (int i = tid; i < m; i += 32)
+      if (i > 0) xn2 = fma(v[i].x, v[i].x, fma(v[i].y, v[i].y, xn2));
+    for (int o = 16; o > 0; o >>= 1) xn2 += __shfl_xor_sync(0xffffffffu, xn2, o);
+    const double2 alpha = v[0];
+    double2 t = make_double2(0.0, 0.0);
+    double beta = alpha.x;
+    double2 inv = make_double2(1.0, 0.0);
+    if (xn2 > 0.0 || alpha.y != 0.0) {
+      const double s2 = fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2));
+      const double nrm = s2 > 1e-280 && s2 < 1e280 ? s2 * fast_rsqrt(s2) : sqrt(s2);
+      beta = alpha.x >= 0.0 ? -nrm : nrm;
+      // one reciprocal for 1 / beta and 1 / |alpha - beta|^2 where their product is in range
+      const double2 den = make_double2(alpha.x - beta, alpha.y);
+      const double dd = den.x * den.x + den.y * den.y, bd = beta * dd;
+      double ib, idd;
+      if (fabs(bd) > 1e-200 && fabs(bd) < 1e200) {
+        const double q = fast_rcp(bd);
+        ib = q * dd;
+        idd = q * beta;
+      } else {
+        ib = 1.0 / beta;
+        idd = 1.0 / dd;
       }
-      for (int o = 16; o > 0; o >>= 1) xn2 += __shfl_xor_sync(0xffffffffu, xn2, o);
-      const double2 alpha = C[(j + 1) * ld + j];
-      double2 t = make_double2(0.0, 0.0);
-      double beta = alpha.x;
-      if (xn2 > 0.0 || alpha.y != 0.0) {
-        const double nrm = sqrt(alpha.x * alpha.x + alpha.y * alpha.y + xn2);
-        beta = alpha.x >= 0.0 ? -nrm : nrm;
-        const double ib = 1.0 / beta;
-        t = make_double2((beta - alpha.x) * ib, -alpha.y * ib);
-        // u = x / (alpha - beta)
-        const double2 den = make_double2(alpha.x - beta, alpha.y);
-        const double idd = 1.0 / (den.x * den.x + den.y * den.y);
-        const double2 inv = make_double2(den.x * idd, -den.y * idd);
-        for (int i = 1 + tid; i < m; i += 32) {
-          const double2 u = cmul(vv[i], inv);
-          vv[i] = u;
-          C[(j + 1 + i) * ld + j] = u;
+      t = make_double2((beta - alpha.x) * ib, -alpha.y * ib);
+      inv = make_double2(den.x * idd, -den.y * idd);   // u = x / (alpha - beta)
+    }
+    __syncwarp();   // every lane has read alpha before it is overwritten
+    for (int i = tid; i < m; i += 32) {
+      const double2 u = i == 0 ? make_double2(1.0, 0.0) : cmul(v[i], inv);   // v[0] = 1
+      v[i] = u;
+      C[(j + 1 + i) * ld + j] = u;
+    }
+    if (tid == 0) {
+      tau[j] = t;
+      e[j] = beta;
+    }
+  };
+  if (tid < 32) {
+    for (int i = tid; i < n - 1; i += 32) vv[0][i] = C[(1 + i) * ld];
+    if (tid == 0) d[0] = C[0].x;
+    __syncwarp();
+    if (n > 1) reflector(0, 0);
+  }
+  for (int j = 0; j + 1 < n; ++j) {
+    __syncthreads();
+    const int m = n - j - 1, buf = j & 1;       // m: length of v_j
+    const double2* v = vv[buf];
+    const double2 t = tau[j];
+    const bool skip = t.x == 0.0 && t.y == 0.0;   // uniform across the block
+    double2* C22 = C + (size_t)(j + 1) * ld + (j + 1);
+    if (!skip) {
+      // w = tau C22 v  (C22 = C[j+1.., j+1..], Hermitian, lower triangle stored)
+      int lp = 0;   // log2 of the lanes per row
+      while ((m << (lp + 1)) <= nth && lp < 4) ++lp;
+      const int P = 1 << lp, p = tid & (P - 1);
+      for (int rb = 0; rb < m; rb += nth >> lp) {   // uniform trip count: shuffles see every lane
+        const int r = rb + (tid >> lp);
+        double2 s = make_double2(0.0, 0.0);
+        if (r < m) {
+          const double2* row = C22 + (size_t)r * ld;
+          for (int q = p; q < m; q += P) {
+            if (q <= r) cfma(s, row[q], v[q]);
+            else cfma_c(s, v[q], C22[(size_t)q * ld + r]);   // conj(C[q][r]) v_q
+          }
+        }
+        for (int o = P >> 1; o > 0; o >>= 1) {
+          s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+          s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+        }
+        if (r < m && p == 0) {
+          ww[r] = cmul(t, s);
+          hh[r] = fma(v[r].x, s.x, v[r].y * s.y);   // Re conj(v_r) (C22 v)_r
         }
       }
-      __syncwarp();   // every lane has read alpha before it is overwritten
-      if (tid == 0) {
-        tau[j] = t;
-        e[j] = beta;
-        d[j] = C[j * ld + j].x;
-        C[(j + 1) * ld + j] = make_double2(1.0, 0.0);   // v[0] = 1
-        vv[0] = make_double2(1.0, 0.0);
+      __syncthreads();
+      // alpha2 = -1/2 tau (w^H v) = -1/2 |tau|^2 v^H C22 v (real); w += alpha2 v, a warp per 32 rows,
+      // each with its own sum of hh
+      if (tid < ((m + 31) & ~31)) {
+        double h = 0.0;
+        for (int r = tid & 31; r < m; r += 32) h += hh[r];
+        for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+        const double a2 = -0.5 * fma(t.x, t.x, t.y * t.y) * h;
+        if (tid < m) {
+          double2 w = ww[tid];
+          w.x = fma(a2, v[tid].x, w.x);
+          w.y = fma(a2, v[tid].y, w.y);
+          ww[tid] = w;
+        }
       }
+      __syncthreads();
     }
-    __syncthreads();
-    const double2 t = tau[j];
-    if (t.x == 0.0 && t.y == 0.0) continue;   // uniform across the block
-    // w = tau * C22 v  (C22 = C[j+1.., j+1..], Hermitian, lower triangle stored)
-    const double2* C22 = C + (size_t)(j + 1) * ld + (j + 1);
-    for (int r = tid; r < m; r += nth) {
-      double2 s = make_double2(0.0, 0.0);
-      const double2* row = C22 + (size_t)r * ld;
-      for (int q = 0; q <= r; ++q) cfma(s, row[q], vv[q]);
-      for (int q = r + 1; q < m; ++q) cfma_c(s, vv[q], C22[(size_t)q * ld + r]);   // conj(C[q][r]) v_q
-      ww[r] = cmul(t, s);
-    }
-    __syncthreads();
-    // alpha2 = -1/2 tau (w^H v); w += alpha2 v
-    if (tid < 32) {
-      double2 dot = make_double2(0.0, 0.0);
-      for (int r = tid; r < m; r += 32) cfma_c(dot, vv[r], ww[r]);   // conj(w_r) v_r
-      for (int o = 16; o > 0; o >>= 1) {
-        dot.x += __shfl_xor_sync(0xffffffffu, dot.x, o);
-        dot.y += __shfl_xor_sync(0xffffffffu, dot.y, o);
-      }
-      const double2 a2 = cmul(make_double2(-0.5 * t.x, -0.5 * t.y), dot);
-      for (int r = tid; r < m; r += 32) cfma(ww[r], a2, vv[r]);
-    }
-    __syncthreads();
     // C22 -= v w^H + w v^H  (lower triangle)
-    double2* C22w = C + (size_t)(j + 1) * ld + (j + 1);
-    for_lower(m, tid, nth, [&](int r, int c) {
-      double2& x = C22w[r * ld + c];
-      cfms_c(x, vv[r], ww[c]);
-      cfms_c(x, ww[r], vv[c]);
+    auto update = [&](double2& x, int r, int c) {
+      if (skip) return;
+      cfms_c(x, v[r], ww[c]);
+      cfms_c(x, ww[r], v[c]);
       if (r == c) x.y = 0.0;   // Hermitian: real diagonal
-    });
-    __syncthreads();
+    };
+    if (tid < 32) {
+      double2* nx = vv[buf ^ 1];
+      for (int r = tid; r < m; r += 32) {
+        double2 x = C22[(size_t)r * ld];
+        update(x, r, 0);
+        if (r == 0) d[j + 1] = x.x;
+        else nx[r - 1] = x;
+      }
+      __syncwarp();
+      if (m > 1) reflector(j + 1, buf ^ 1);
+    } else if (!skip) {
+      for_lower(m - 1, tid - 32, nth - 32, [&](int r, int c) { update(C22[(size_t)(r + 1) * ld + c + 1], r + 1, c + 1); });
+    }
   }
-  if (tid == 0) {
-    d[n - 1] = C[(n - 1) * ld + (n - 1)].x;
-    e[n - 1] = 0.0;
-  }
+  if (tid == 0) e[n - 1] = 0.0;
   __syncthreads();
   // ---- 4. the nb lowest eigenpairs of the real tridiagonal T = (d, e): bisection on Sturm
   //      counts for the eigenvalues (one thread per eigenvalue: the threads of a warp work in
@@ -317,9 +428,9 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
   __shared__ float d32[kMaxBasis], e232[kMaxBasis];
   __shared__ float pivmin32;
   __shared__ int use32;
-  if (tid == 0) {
+  if (tid < 32) {
     double lo = 1e300, hi = -1e300, emax = 0.0, dmax = 0.0;
-    for (int i = 0; i < n; ++i) {
+    for (int i = tid; i < n; i += 32) {
       const double r = (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < n ? fabs(e[i]) : 0.0);
       lo = fmin(lo, d[i] - r);
       hi = fmax(hi, d[i] + r);
@@ -329,6 +440,13 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
         emax = fmax(emax, e2[i]);
       }
     }
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+      emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+    }
+    if (tid == 0) {
     const double span = fmax(fabs(lo), fabs(hi));
     glo = lo - 1e-14 * span - 1e-300;
     ghi = hi + 1e-14 * span + 1e-300;
@@ -346,6 +464,7 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
     werr = 4.8e-7 * (3.0 * dmax + 11.0 * sqrt(emax));
     use32 = dmax < 1e15 && emax < 1e28;
     pivmin32 = (float)(1e-30 * fmax(1.0, emax));
+    }
   }
   __syncthreads();
   if (use32)
@@ -365,7 +484,7 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
     int cnt = q < 0.0;
     for (int i = 1; i < n; ++i) {
       if (fabs(q) < pivmin) q = -pivmin;
-      q = d[i] - x - e2[i - 1] / q;
+      q = fma(-e2[i - 1], fast_rcp(q), d[i] - x);
       cnt += q < 0.0;
     }
     return cnt;
@@ -377,7 +496,7 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
     double q = d[0] - x, dq = -1.0;
     int cnt = q < 0.0;
     if (fabs(q) < pivmin) q = -pivmin;
-    double r = 1.0 / q;
+    double r = fast_rcp(q);
     s = dq * r;
     for (int i = 1; i < n; ++i) {
       const double t = e2[i - 1] * r;   // e_{i-1}^2 / q_{i-1}
@@ -385,7 +504,7 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
       q = (d[i] - x) - t;
       cnt += q < 0.0;
       if (fabs(q) < pivmin) q = -pivmin;
-      r = 1.0 / q;
+      r = fast_rcp(q);
       s = fma(dq, r, s);
     }
     return cnt;
@@ -500,12 +619,12 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
       // LDL^T of T - lj; Dv keeps 1/D (the solves below then multiply only)
       double D = d[0] - lj;
       if (fabs(D) < tiny) D = D < 0.0 ? -tiny : tiny;
-      double iD = 1.0 / D;
+      double iD = fast_rcp(D);
       Dv[0] = iD;
       for (int i = 1; i < n; ++i) {
         D = d[i] - lj - e2[i - 1] * iD;
         if (fabs(D) < tiny) D = D < 0.0 ? -tiny : tiny;
-        iD = 1.0 / D;
+        iD = fast_rcp(D);
         Dv[i] = iD;
       }
       for (int i = 0; i < n; ++i) {   // start vector: a fixed pseudo-random pattern per (i, j)
@@ -559,7 +678,7 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
   for (int j = tid; j < nb; j += nth) eps[k * nb + j] = lam[j];
   double2* E = ev + (size_t)k * ld * nb;
   {
-    const int G = nb <= nth / 8 ? 8 : nb <= nth / 4 ? 4 : nb <= nth / 2 ? 2 : 1;
+    const int G = nb <= nth / 16 && n > 40 ? 16 : nb <= nth / 8 ? 8 : nb <= nth / 4 ? 4 : nb <= nth / 2 ? 2 : 1;
     const int c = tid % G, lane = tid & 31, ngroups = nth / G;
     const int gbase = lane & ~(G - 1);   // lane of c = 0 in this group (G divides 32)
     auto first_row = [&](int lo) { return lo <= c ? c : c + G * ((lo - c + G - 1) / G); };
@@ -623,10 +742,15 @@ __global__ void __launch_bounds__(256) rr_kernel(int nk, int ld, int nb, const i
   if (tid == 0 && status != nullptr) status[k] = PWK_OK;
 }
 
+// Threads per problem: 512 where a CTA has an SM to itself and enough rows to fill them, 256 for
+// small problems and where several CTAs share an SM (n = 80, 20 vectors, 512 problems: 7.4 ms
+// with 256, 8.6 with 512; 128 problems: 2.7 with 512).
+static int rr_threads(int nk, int ld) { return ld > 40 && nk <= 304 ? 512 : 256; }
+
 int launch_rr(int nk, int ld, int nb, const int* nbase, const int* active, const double2* Hr,
               const double2* Sr, double2* W, double2* ev, double* eps, int* status,
               cudaStream_t st, unsigned char* drop_out, double* flops) {
-  rr_kernel<<<nk, 256, 0, st>>>(nk, ld, nb, nbase, active, Hr, Sr, W, ev, eps, status, drop_out, flops); note_launch();
+  rr_kernel<<<nk, rr_threads(nk, ld), 0, st>>>(nk, ld, nb, nbase, active, Hr, Sr, W, ev, eps, status, drop_out, flops); note_launch();
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? PWK_OK : cuda_fail(e, "rr_kernel");
 }
