@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "fft_line.cuh"
+#include "fixed_block.cuh"
 #include "fused_kernel.cuh"
 #include "pwk_internal.h"
 #include "solvers.h"
@@ -42,16 +43,32 @@ struct DrhoArgs {
   int nstick_max = 0, m1lo = 0, P = 0, L = 0, zs = 0;
 };
 
+// CTAs per SM the registers allow for: an FP64 line of N <= 20 fits 128 registers
 template <typename T, int N>
-__global__ void __launch_bounds__(256) drho_kernel(DrhoArgs a) {
+constexpr int drho_ctas() { return sizeof(T) == 4 || N <= 20 ? 2 : 1; }
+
+template <typename V>
+__device__ __forceinline__ V drho_value(float2 q) { return q; }
+template <typename V>
+__device__ __forceinline__ V drho_value(longlong2 q) { return V{__ll2double_rn(q.x), __ll2double_rn(q.y)}; }
+
+// FP64 transforms run in the fixed point of fixed.cuh (inverse only, so each field keeps the one
+// scale of its vector); the values come back to double at the product.  768 pairs at N = 20: 1.05
+// ms with FP64 transforms, 0.43 with these; then bound by the product (ten FP64 instructions per
+// grid point, 57 % of that pipe) and the barriers between the passes.
+template <typename T, int N>
+__global__ void __launch_bounds__(256, drho_ctas<T, N>()) drho_kernel(DrhoArgs a) {
   using V = c2_t<T>;
+  using A = fft_arith_t<T>;
+  using VA = c2_t<A>;
+  constexpr bool FX = std::is_same<A, long long>::value;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int zs = a.zs, P = a.P, L = a.L;
-  V* ZA = reinterpret_cast<V*>(smem_raw);                  // [nstick_max][zs]  u
-  V* ZB = ZA + (size_t)a.nstick_max * zs;                  // [nstick_max][zs]  du
-  V* YA = ZB + (size_t)a.nstick_max * zs;                  // [P][N][L]
-  V* YB = YA + (size_t)P * N * L;
-  V* XA = YB + (size_t)P * N * L;                          // [N (l1)][N (l2)][L]
+  VA* ZA = reinterpret_cast<VA*>(smem_raw);                // [nstick_max][zs]  u
+  VA* ZB = ZA + (size_t)a.nstick_max * zs;                 // [nstick_max][zs]  du
+  VA* YA = ZB + (size_t)a.nstick_max * zs;                 // [P][N][L]
+  VA* YB = YA + (size_t)P * N * L;
+  V* XA = reinterpret_cast<V*>(YB + (size_t)P * N * L);    // [N (l1)][N (l2)][L]
   short* sid = reinterpret_cast<short*>(XA + (size_t)N * N * L);   // [P][N]
   const int tid = threadIdx.x, nth = blockDim.x;
   double2* acc = a.part + (size_t)blockIdx.x * N * N * N;
@@ -61,37 +78,55 @@ __global__ void __launch_bounds__(256) drho_kernel(DrhoArgs a) {
     const int k = pr / a.nocc, v = pr - k * a.nocc;
     const int ns = a.nstick[k];
     const int nka = a.npwk[k], nkb = a.npwq[k];
-    const double wk = 4.0 * a.w[k];
+    double wk = 4.0 * a.w[k];
+    const double2* pu = static_cast<const double2*>(a.uk) + ((size_t)k * a.nocc + v) * a.npw_k;
+    const double2* pd = a.du + ((size_t)k * a.nocc + v) * a.npw_kq;
     __syncthreads();   // the previous pair is done with the buffers
-    for (int i = tid; i < ns * zs; i += nth) ZA[i] = ZB[i] = V{T(0), T(0)};
+    for (int i = tid; i < ns * zs; i += nth) ZA[i] = ZB[i] = VA{A(0), A(0)};
     {
       const short* sk = a.sid + (size_t)k * P * N;
       for (int i = tid; i < P * N; i += nth) sid[i] = sk[i];
     }
+    FxScale su{1.0, 0.0, 0, false}, sd = su;
+    int shift_u = 0;   // exponent taken into u at the product (0 unless the pair's is extreme)
+    if constexpr (FX) {
+      FxScratch* scratch = fx_scratch_at(reinterpret_cast<unsigned char*>(sid + P * N));
+      su = fx_block_scale(pu, nka, scratch);
+      __syncthreads();
+      sd = fx_block_scale(pd, nkb, scratch);
+      const int e = -su.exp - sd.exp;
+      if (fx_plain_scale(e)) {
+        wk = fx_factor(wk, e);
+      } else {
+        wk = ldexp(wk, -sd.exp);
+        shift_u = -su.exp;
+      }
+      if (su.bad || sd.bad) wk = __longlong_as_double(0x7ff8000000000000LL);
+    }
     __syncthreads();
     {
-      const double2* pu = static_cast<const double2*>(a.uk) + ((size_t)k * a.nocc + v) * a.npw_k;
-      const double2* pd = a.du + ((size_t)k * a.nocc + v) * a.npw_kq;
       const int* gi = a.gin + (size_t)k * a.npw_k;
       const int* go = a.gout + (size_t)k * a.npw_kq;
       for (int g = tid; g < nka; g += nth) {
         const int m = gi[g];
         const double2 c = pu[g];
-        ZA[(m >> 8) * zs + (m & 255)] = V{T(c.x), T(c.y)};
+        if constexpr (FX) ZA[(m >> 8) * zs + (m & 255)] = fx_from(su, c);
+        else ZA[(m >> 8) * zs + (m & 255)] = VA{A(c.x), A(c.y)};
       }
       for (int g = tid; g < nkb; g += nth) {
         const int m = go[g];
         const double2 c = pd[g];
-        ZB[(m >> 8) * zs + (m & 255)] = V{T(c.x), T(c.y)};
+        if constexpr (FX) ZB[(m >> 8) * zs + (m & 255)] = fx_from(sd, c);
+        else ZB[(m >> 8) * zs + (m & 255)] = VA{A(c.x), A(c.y)};
       }
     }
     __syncthreads();
     // inverse z transforms of both fields on the sticks (Eq. zfft)
     for (int s = tid; s < 2 * ns; s += nth) {
-      V x[N];
-      V* zr = (s < ns ? ZA + s * zs : ZB + (s - ns) * zs);
+      VA x[N];
+      VA* zr = (s < ns ? ZA + s * zs : ZB + (s - ns) * zs);
       PWK_SFOR(N, j, x[j] = zr[j]);
-      LineFFT<T, N, +1>::run(x);
+      LineFFT<A, N, +1>::run(x);
       PWK_SFOR(N, j, zr[j] = x[OutSlot<N, j>::value]);
     }
     __syncthreads();
@@ -101,62 +136,76 @@ __global__ void __launch_bounds__(256) drho_kernel(DrhoArgs a) {
       for (int t = tid; t < 2 * P * lc; t += nth) {
         const int f = t / (P * lc), r = t - f * P * lc;
         const int p = r / lc, c = r - p * lc;
-        const V* Z = f ? ZB : ZA;
-        V x[N];
+        const VA* Z = f ? ZB : ZA;
+        VA x[N];
         PWK_SFOR(N, j, {
           const int s = sid[p * N + j];
-          x[j] = s >= 0 ? Z[s * zs + l0 + c] : V{T(0), T(0)};
+          x[j] = s >= 0 ? Z[s * zs + l0 + c] : VA{A(0), A(0)};
         });
-        LineFFT<T, N, +1>::run(x);
-        V* yp = (f ? YB : YA) + (size_t)p * N * L + c;
+        LineFFT<A, N, +1>::run(x);
+        VA* yp = (f ? YB : YA) + (size_t)p * N * L + c;
         PWK_SFOR(N, l2, yp[l2 * L] = x[OutSlot<N, l2>::value]);
       }
       __syncthreads();
-      // x lines (Eq. xfft) of u, kept in shared memory
-      for (int t = tid; t < N * lc; t += nth) {
-        const int l2 = t / lc, c = t - l2 * lc;
-        V x[N];
-        PWK_SFOR(N, i, {
-          const int p = plane_of_slot<N>(i, a.m1lo);
-          x[i] = (unsigned)p < (unsigned)P ? YA[((size_t)p * N + l2) * L + c] : V{T(0), T(0)};
-        });
-        LineFFT<T, N, +1>::run(x);
-        PWK_SFOR(N, l1, XA[((size_t)l1 * N + l2) * L + c] = x[OutSlot<N, l1>::value]);
-      }
-      __syncthreads();
-      // x lines of du, product conj(u) du added to this CTA's grid
-      for (int t = tid; t < N * lc; t += nth) {
-        const int l2 = t / lc, c = t - l2 * lc;
-        V x[N];
-        PWK_SFOR(N, i, {
-          const int p = plane_of_slot<N>(i, a.m1lo);
-          x[i] = (unsigned)p < (unsigned)P ? YB[((size_t)p * N + l2) * L + c] : V{T(0), T(0)};
-        });
-        LineFFT<T, N, +1>::run(x);
-        double2* ag = acc + (size_t)l2 * N + l0 + c;
-        PWK_SFOR(N, l1, {
-          const V ua = XA[((size_t)l1 * N + l2) * L + c], ub = x[OutSlot<N, l1>::value];
-          const double re = (double)ua.x * ub.x + (double)ua.y * ub.y;   // conj(u) du
-          const double im = (double)ua.x * ub.y - (double)ua.y * ub.x;
-          double2& d = ag[(size_t)l1 * N * N];
-          d.x += wk * re;
-          d.y += wk * im;
-        });
+      // x lines (Eq. xfft): those of u kept in shared memory, then those of du with the product
+      // conj(u) du added to this CTA's grid
+      for (int f = 0; f < 2; ++f) {
+        const VA* Y = f ? YB : YA;
+        for (int t = tid; t < N * lc; t += nth) {   // the same thread takes a line of both fields
+          const int l2 = t / lc, c = t - l2 * lc;
+          VA x[N];
+          PWK_SFOR(N, i, {
+            const int p = plane_of_slot<N>(i, a.m1lo);
+            x[i] = (unsigned)p < (unsigned)P ? Y[((size_t)p * N + l2) * L + c] : VA{A(0), A(0)};
+          });
+          LineFFT<A, N, +1>::run(x);
+          V* xa = XA + (size_t)l2 * L + c;
+          if (f == 0) {
+            PWK_SFOR(N, l1, {
+              V z = drho_value<V>(x[OutSlot<N, l1>::value]);
+              if constexpr (FX) {
+                if (shift_u != 0) z = V{ldexp(z.x, shift_u), ldexp(z.y, shift_u)};   // uniform
+              }
+              xa[(size_t)l1 * N * L] = z;
+            });
+          } else {
+            double2* ag = acc + (size_t)l2 * N + l0 + c;
+            PWK_SFOR(N, l1, {
+              const V ua = xa[(size_t)l1 * N * L], ub = drho_value<V>(x[OutSlot<N, l1>::value]);
+              const double re = (double)ua.x * ub.x + (double)ua.y * ub.y;   // conj(u) du
+              const double im = (double)ua.x * ub.y - (double)ua.y * ub.x;
+              double2& d = ag[(size_t)l1 * N * N];
+              d.x += wk * re;
+              d.y += wk * im;
+            });
+          }
+        }
       }
       __syncthreads();
     }
   }
 }
 
-// drho[l] = sum_p part[p][l] in ascending p
-__global__ void drho_reduce_kernel(int nr, int nparts, const double2* part, double2* out) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= nr) return;
+// (One thread per point left most SMs idle: 57 us for 256 grids of 20^3, 15 with this split.)
+// drho[l] = sum_p part[p][l]: 32 points per CTA, each of its 8 warps sums every eighth partial
+// grid in ascending order, and the eight sums are added in ascending order.
+__global__ void __launch_bounds__(256) drho_reduce_kernel(int nr, int nparts, const double2* part, double2* out) {
+  __shared__ double2 sums[8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int l = blockIdx.x * 32 + lane;
   double sx = 0.0, sy = 0.0;
-  for (int p = 0; p < nparts; ++p) {
-    const double2 v = part[(size_t)p * nr + l];
-    sx += v.x;
-    sy += v.y;
+  if (l < nr)
+    for (int p = warp; p < nparts; p += 8) {
+      const double2 v = part[(size_t)p * nr + l];
+      sx += v.x;
+      sy += v.y;
+    }
+  sums[warp][lane] = make_double2(sx, sy);
+  __syncthreads();
+  if (warp != 0 || l >= nr) return;
+  for (int w = 1; w < 8; ++w) {
+    sx += sums[w][lane].x;
+    sy += sums[w][lane].y;
   }
   out[l] = make_double2(sx, sy);
 }
@@ -331,7 +380,7 @@ extern "C" int pwk_drho_batched(pwk_plan* pq, pwk_plan* pk, int precision, const
                                : launch_drho_typed<float>(N, a, nparts, smem, st);
   }
   if (rc == PWK_OK) {
-    drho_reduce_kernel<<<(int)((nr + 255) / 256), 256, 0, st>>>((int)nr, nparts, part,
+    drho_reduce_kernel<<<(int)((nr + 31) / 32), 256, 0, st>>>((int)nr, nparts, part,
                                                                 static_cast<double2*>(drho)); note_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) rc = cuda_fail(e, "drho_reduce_kernel");
