@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(256, drho_ctas<T, N>()) drho_kernel(DrhoArgs a
       const short* sk = a.sid + (size_t)k * P * N;
       for (int i = tid; i < P * N; i += nth) sid[i] = sk[i];
     }
-    FxScale su{1.0, 0.0, 0, false}, sd = su;
+    FxScale su{1.0, 0.0, 0, false, 0}, sd = su;
     int shift_u = 0;   // exponent taken into u at the product (0 unless the pair's is extreme)
     if constexpr (FX) {
       FxScratch* scratch = fx_scratch_at(reinterpret_cast<unsigned char*>(sid + P * N));

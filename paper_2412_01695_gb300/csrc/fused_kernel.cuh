@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
     const short* sk = a.sid + (size_t)k * P * N;
     for (int i = tid; i < P * N; i += nth) sid[i] = sk[i];
   }
-  FxScale scale{1.0, 0.0, 0, false};
+  FxScale scale{1.0, 0.0, 0, false, 0};
   if constexpr (FX) {
     scale = fx_block_scale(pin, npi, fx_scratch_at(sz + a.nstick_max));   // synchronises the block
   } else {
@@ -141,12 +141,25 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
     }
   }
   const V* nl_bk = nl ? static_cast<const V*>(a.beta) + (size_t)k * a.nkb * a.npw_beta : nullptr;
+  // FP64: the integer form, with beta and C turned into limbs where they are used
+  [[maybe_unused]] const int* be = nl && FX ? a.bexp + (size_t)k * a.nkb : nullptr;
+  [[maybe_unused]] int* ex = reinterpret_cast<int*>(nls + 3 * (size_t)a.nkb);
+  [[maybe_unused]] auto load_b = [&](int m, int g) {
+    const V b = nl_bk[(size_t)m * a.npw_beta + g];
+    return nl_limbs(double2{b.x, b.y}, be[m] == kFxBadField ? 0 : be[m]);
+  };
   if constexpr (nl) {
-    if constexpr (FX) nl_fused_project<T>(a, nl_bk, a.npw_beta, pin, npi, nls);
-    else nl_fused_project<T>(a, nl_bk, a.npw_beta, psis, npi, nls);
+    if constexpr (FX)
+      nl_fx_project(a.nkb, npi, be, scale.top, load_b, [&](int g) { return nl_limbs(pin[g], scale.top); }, nls);
+    else
+      nl_fused_project<T>(a, nl_bk, a.npw_beta, psis, npi, nls);
   }
   __syncthreads();
   if (nl) nl_fused_coef<T>(a, nls);   // read after the barriers that follow
+  if constexpr (nl && FX) {
+    __syncthreads();
+    nl_fx_coef(a.nkb, a.sout != nullptr && a.qm != nullptr, be, nls, ex);
+  }
 
   // ---- 2: inverse z transforms on the sticks
   for (int s = tid; s < ns; s += nth) {
@@ -270,13 +283,18 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
           acc.y += t2 * c.y;
         }
         if constexpr (nl) {   // the in and out spheres are the same here (npi == npo)
+          const bool with_q = with_s && a.qm != nullptr;
           V h, sv;
-          nl_fused_addback<T>(a, nl_bk, a.npw_beta, g, nls, with_s && a.qm != nullptr, h, sv);
+          if constexpr (FX) {
+            nl_fx_addback(a.nkb, g, reinterpret_cast<const int4*>(nls) + a.nkb, ex, with_q, load_b, h, sv);
+          } else {
+            nl_fused_addback<T>(a, nl_bk, a.npw_beta, g, nls, with_q, h, sv);
+          }
           acc.x += h.x;
           acc.y += h.y;
           if (with_s) {
             const VI cv = pin[g];
-            sout[g] = a.qm != nullptr ? VI{cv.x + TI(sv.x), cv.y + TI(sv.y)} : cv;
+            sout[g] = with_q ? VI{cv.x + TI(sv.x), cv.y + TI(sv.y)} : cv;
           }
         }
       }

@@ -188,6 +188,20 @@ __global__ void fx_field_kernel(int N, int ncomp, const double* in, const unsign
   }
 }
 
+// Exponents of the projectors, a warp each: every |component| < 2^exponent (kFxBadField: one is
+// not finite)
+__global__ void beta_exponent_kernel(int n, int npw_max, const double2* beta, int* bexp) {
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= n) return;   // uniform over the warp
+  unsigned h = 0;
+  for (int g = lane; g < npw_max; g += 32) {
+    const double2 b = beta[(size_t)i * npw_max + g];
+    h = max(h, max((unsigned)__double2hiint(b.x) & 0x7fffffffu, (unsigned)__double2hiint(b.y) & 0x7fffffffu));
+  }
+  h = __reduce_max_sync(0xffffffffu, h);
+  if (lane == 0) bexp[i] = (h >> 20) == 0x7ff ? kFxBadField : (int)(h >> 20) - 1022;
+}
+
 // sum of n values by one CTA in a fixed order (the result is the same on every run)
 __global__ void sum_kernel(size_t n, const double* in, double* out) {
   __shared__ double sh[256];
@@ -414,6 +428,7 @@ static void set_fused_nl(const pwk_plan* p, int precision, FusedArgs& a, void* s
   a.Dm = f64 ? static_cast<const void*>(p->d_D) : static_cast<const void*>(p->d_D32);
   a.qm = f64 ? static_cast<const void*>(p->d_q) : static_cast<const void*>(p->d_q32);
   a.sout = sout;
+  a.bexp = p->d_bexp;
   a.nkb = p->nkb;
   a.npw_beta = p->npw_max;
   fused_layout(p, precision, s, &a.nl_off, &a.loc_off);
@@ -583,10 +598,14 @@ int autotune_shape(pwk_plan* p, int precision) {
         ts = std::min(ts, split(false));
         if (try_tc) tt = std::min(tt, split(true));
       }
-      // the separate CUDA-core kernels unless another path is faster by more than 3 %: near
-      // ties (timing noise) then resolve the same way in every process
-      const float best_other = std::min(tf, tt);
-      if (best_other < 0.97f * ts) {
+      // near ties (timing noise) resolve the same way in every process: FP32 takes the separate
+      // CUDA-core kernels unless another path is faster by more than 3 %.  FP64 takes the fused
+      // terms unless the separate kernels are: those hold the FP64 pipe, and on uneven lists with
+      // S they cost twice what this sample of whole band sets shows (H and S of 237 items at N =
+      // 27 with 8 projectors: 0.66 ms separate, 0.27 to 0.36 fused)
+      if (precision == PWK_FP64) {
+        fused = tf <= 1.03f * ts;
+      } else if (std::min(tf, tt) < 0.97f * ts) {
         fused = tf <= tt;
         tc = !fused;
       }
@@ -996,6 +1015,9 @@ int pwk_plan_create(pwk_plan** out, const double* A, int N1, int N2, int N3, int
     TRY(plan_alloc(p, (void**)&p->d_beta32, sizeof(float) * nb2));
     to_f32_kernel<<<blocks_for(nb2), 256>>>(nb2, static_cast<const double*>(beta), (float*)p->d_beta32); note_launch();
     TRYC(cudaGetLastError(), "beta to f32");
+    TRY(plan_alloc(p, (void**)&p->d_bexp, sizeof(int) * (size_t)nk * nkb));
+    beta_exponent_kernel<<<blocks_for((size_t)nk * nkb, 8), 256>>>(nk * nkb, npw_max, static_cast<const double2*>(beta), p->d_bexp); note_launch();
+    TRYC(cudaGetLastError(), "beta_exponent_kernel");
     std::vector<float> D32(p->h_D.begin(), p->h_D.end());
     TRY(plan_alloc(p, (void**)&p->d_D, sizeof(double) * nkb * nkb));
     TRY(plan_alloc(p, (void**)&p->d_D32, sizeof(float) * nkb * nkb));

@@ -90,6 +90,7 @@ struct pwk_plan {
   double* d_g2 = nullptr;        // [nk][npw_max] |k+G|^2
   const double2* d_beta = nullptr;   // caller-owned
   float2* d_beta32 = nullptr;
+  int* d_bexp = nullptr;         // [nk][nkb] every |component of beta_m(k)| < 2^exponent (fixed.cuh)
   double* d_D = nullptr;
   float* d_D32 = nullptr;
   double* d_q = nullptr;          // overlap coefficients q_mn (null: S = 1), pwk_plan_set_overlap
@@ -160,6 +161,7 @@ struct FusedArgs {
   int* err = nullptr;
   // nonlocal projector terms fused into the kernel (nl_fused.cuh); beta == null: none
   const void* beta = nullptr;      // [nk][nkb][npw_beta] complex of the arithmetic type
+  const int* bexp = nullptr;       // FP64: [nk][nkb] exponents of the projectors
   const void* Dm = nullptr;        // [nkb][nkb] real of the arithmetic type
   const void* qm = nullptr;        // [nkb][nkb] or null (S = 1)
   void* sout = nullptr;            // S C output (io type) or null
