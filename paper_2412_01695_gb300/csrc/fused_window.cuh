@@ -5,12 +5,15 @@
 // W = N/4: a grid chosen to hold the differences G - G' of the basis (Sec. 4: "N_i large
 // enough"), N >= 4 max|m|, always satisfies it.  With the window known at compile time:
 //   * the z-sticks live in a dense (2W+1) x (2W+1) square of rows [m1][m2] (rows without a
-//     stick of this k stay zero), so the y pass reads and writes them without a stick table;
+//     stick of this k stay zero), so the y pass reads and writes them without a stick table; on
+//     grids of N >= 30 (window_lists) they lie one row after another instead, m1 fastest, found
+//     from the y pass by a table over the window (a row of zeros stands for a missing stick):
+//     half the square is empty there, and the shared memory it takes costs a CTA per SM;
 //   * every transform reads only the 2W+1 window inputs (the others are literal zeros) and
 //     stores only the outputs that are used later; no per-element index arithmetic or
 //     predicated shared-memory access remains.
-// The real sticks of the k-point (for the z passes) and the packed (row, m3) place of every
-// basis vector come from the plan's window tables.
+// The rows of the sticks (or the table) and the packed (row, m3) place of every basis vector
+// come from the plan's window tables.
 #pragma once
 #include <type_traits>
 
@@ -66,29 +69,45 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
   const int ns = a.nstick[k];
   const int zs = a.zs, L = a.L, yps = a.yps;
 
-  using U = VA;
-  U* Z = reinterpret_cast<U*>(smem_raw);               // [NW*NW][zs]
-  // fixed point: the shifts of the z lines next to the square (the gather reads them while the
+  constexpr bool LIST = window_lists(N);
+  const int nz = a.nstick_max;                          // LIST: the row of zeros
+  const int nrows = LIST ? nz + 1 : NW * NW;
+  VA* Z = reinterpret_cast<VA*>(smem_raw);              // [nrows][zs]
+  // fixed point: the shifts of the z lines next to the sticks (the gather reads them while the
   // projector terms reuse what follows), those of the x lines [ycopies][N][L] and y lines
   // [NW][N] at the end
-  unsigned char* sz = reinterpret_cast<unsigned char*>(Z + (size_t)NW * NW * zs);   // [NW*NW]
-  U* Y = Z + (size_t)NW * NW * zs + (FX ? window_shift_elems(NW) : 0);   // [NW][yps] (N x L used per plane)
-  // plane buffers: one [NW][yps] for the CTA (MODE 0) or one per warp (MODE 1), then the rows
+  unsigned char* sz = reinterpret_cast<unsigned char*>(Z + (size_t)nrows * zs);   // [nrows]
+  VA* Y = Z + (size_t)nrows * zs + (FX ? window_shift_elems(nrows) : 0);   // [NW][yps] (N x L used per plane)
+  // plane buffers: one [NW][yps] for the CTA (MODE 0) or one per warp (MODE 1), then the rows of
+  // the sticks, or the table [NW (m2)][NW (m1)]
   const int ycopies = MODE == 1 ? (int)(blockDim.x >> 5) : 1;
-  short* rows = reinterpret_cast<short*>(Y + (size_t)ycopies * NW * yps);  // [nstick_max]
-  unsigned char* sx = reinterpret_cast<unsigned char*>(rows + a.nstick_max);
+  short* tab = reinterpret_cast<short*>(Y + (size_t)ycopies * NW * yps);
+  unsigned char* sx = reinterpret_cast<unsigned char*>(tab + (LIST ? NW * NW : nz));
   unsigned char* sy = sx + (size_t)ycopies * N * L;
+  auto stick_row = [&](int s) { return LIST ? s : (int)tab[s]; };
+  auto window_row = [&](int p, int i) { return LIST ? (int)tab[i * NW + p] : p * NW + i; };   // plane p, m2 index i
 
   const VI* pin = static_cast<const VI*>(a.in) + ((size_t)k * a.nvec_in + vin) * a.npw_in_max;
   VI* pout = static_cast<VI*>(a.out) + ((size_t)k * a.nvec_out + vout) * a.npw_out_max;
 
   // C(G) is read from global memory by the two stages that need it (scatter, kinetic term):
   // the second read hits L1/L2, and the shared memory a staged copy would take buys occupancy.
-  // ---- 0: zero the stick square, stage the stick rows
-  for (int i = tid; i < NW * NW * zs; i += nth) Z[i] = U{};
-  {
-    const short* rk = a.sid + (size_t)k * a.nstick_max;
-    for (int i = tid; i < ns; i += nth) rows[i] = rk[i];
+  // ---- 0: zero the rows, stage the table
+  for (int i = tid; i < (LIST ? ns : nrows) * zs; i += nth) Z[i] = VA{A(0), A(0)};
+  if constexpr (LIST) {
+    for (int i = tid; i < zs; i += nth) Z[(size_t)nz * zs + i] = VA{A(0), A(0)};
+    const short* rk = a.sid + (size_t)k * NW * NW;
+    for (int i = tid; i < NW * NW; i += nth) {
+      const int r = rk[i];
+      tab[i] = (short)(r < 0 ? nz : r);
+      if (FX && r >= 0) sz[r] = (unsigned char)(i % NW);   // the stick's m1 plane, until its shift
+    }
+  } else {
+    const short* rk = a.sid + (size_t)k * nz;
+    for (int i = tid; i < ns; i += nth) {
+      tab[i] = rk[i];
+      if (FX) sz[rk[i]] = (unsigned char)(rk[i] / NW);
+    }
   }
   FxScale scale{1.0, 0.0, 0, false, 0};
   if constexpr (FX) {
@@ -114,7 +133,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
   // are its own.
   const int warp = MODE == 1 ? tid >> 5 : 0, nw = MODE == 1 ? nth >> 5 : 1;
   const int lane0 = MODE == 1 ? tid & 31 : tid, step0 = MODE == 1 ? 32 : nth;
-  U* Yc = Y + (size_t)warp * NW * yps;        // [NW][yps]: plane p row, (l2, cc) at l2 L + cc
+  VA* Yc = Y + (size_t)warp * NW * yps;        // [NW][yps]: plane p row, (l2, cc) at l2 L + cc
   auto sync_pass = [&]() {
     if constexpr (MODE == 1) __syncwarp();
     else __syncthreads();
@@ -122,7 +141,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
   if constexpr (!FX) {
     for (int s = tid; s < ns; s += nth) {
       VA x[N];
-      VA* zr = Z + rows[s] * zs;
+      VA* zr = Z + stick_row(s) * zs;
       PWK_SFOR(N, j, x[j] = Wn::in(j) ? zr[j] : VA{A(0), A(0)});
       LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
       PWK_SFOR(N, j, zr[j] = x[OutSlot<N, j>::value]);
@@ -131,10 +150,13 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     for (int l0 = warp * L; l0 < N; l0 += nw * L) {
       const int lc = min(L, N - l0);
       for (int t = lane0; t < NW * lc; t += step0) {
-        const int c = t / NW, p = t - c * NW;   // plane fastest: conflict-free (see window_strides)
+        const int c = t / NW, p = t - c * NW;   // plane fastest: see window_strides
         VA x[N];
-        const VA* zp = Z + (size_t)p * NW * zs + l0 + c;
-        PWK_SFOR(N, j, x[j] = Wn::in(j) ? zp[Wn::idx(j) * zs] : VA{A(0), A(0)});
+        const VA* zp = Z + l0 + c;
+        PWK_SFOR(N, j, {
+          if constexpr (Wn::in(j)) x[j] = zp[window_row(p, Wn::idx(j)) * zs];
+          else x[j] = VA{A(0), A(0)};
+        });
         LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
         VA* yp = Yc + (size_t)p * yps + c;
         PWK_SFOR(N, l2, yp[l2 * L] = x[OutSlot<N, l2>::value]);
@@ -165,9 +187,12 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
         const VA* yp = Yc + (size_t)p * yps + c;
         PWK_SFOR(N, l2, x[l2] = yp[l2 * L]);
         LineFFT<A, N, -1>::run(x);
-        VA* zp = Z + (size_t)p * NW * zs + l0 + c;
+        VA* zp = Z + l0 + c;
         PWK_SFOR(N, j, {
-          if constexpr (Wn::in(j)) zp[Wn::idx(j) * zs] = x[OutSlot<N, j>::value];
+          if constexpr (Wn::in(j)) {
+            const int row = window_row(p, Wn::idx(j));
+            if (!LIST || row != nz) zp[row * zs] = x[OutSlot<N, j>::value];
+          }
         });
       }
       sync_pass();
@@ -175,7 +200,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     __syncthreads();
     for (int s = tid; s < ns; s += nth) {
       VA x[N];
-      VA* zr = Z + rows[s] * zs;
+      VA* zr = Z + stick_row(s) * zs;
       PWK_SFOR(N, j, x[j] = zr[j]);
       LineFFT<A, N, -1>::run(x);
       PWK_SFOR(N, j, {
@@ -186,40 +211,46 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     // fixed point: one copy of the inverse and of the forward code for the z and y lines
     // (unrolled over a line it is thousands of instructions, and the instruction cache holds
     // few): stages -1 (inverse z), a chunk's y, x, y each, N (forward z).
-    // A window line reads its m >= 0 part from `pos` and its m < 0 part from `neg` (both at m
-    // times the stride).
+    // z: the line is stick t; y: plane t % NW of column l0 + t / NW, its window elements in the
+    // rows of the table.
     unsigned char* sxc = sx + (size_t)warp * N * L;
-    // plane fastest over the threads of a y pass: conflict-free (see window_strides)
-    auto y_square = [&](int t, int l0) { return Z + ((size_t)(t % NW) * NW + W) * zs + l0 + t / NW; };
-    auto y_chunk = [&](int t) { return Yc + (size_t)(t % NW) * yps + t / NW; };
-    auto inverse_line = [&](const VA* pos, const VA* neg, int stride, VA* out, int ostride) {
+    auto inverse_line = [&](bool z, int t, int l0) {
       VA x[N];
+      VA* zp = z ? Z + stick_row(t) * zs : Z + l0 + t / NW;
       PWK_SFOR(N, j, {
-        if constexpr (!Wn::in(j)) x[j] = VA{A(0), A(0)};
-        else if constexpr (j <= W) x[j] = pos[j * stride];
-        else x[j] = neg[(j - N) * stride];
+        if constexpr (!Wn::in(j)) {
+          x[j] = VA{A(0), A(0)};
+        } else {
+          const int o = z ? j : window_row(t % NW, Wn::idx(j)) * zs;
+          x[j] = zp[o];
+        }
       });
       LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
-      PWK_SFOR(N, j, out[j * ostride] = x[OutSlot<N, j>::value]);
+      VA* out = z ? zp : Yc + (size_t)(t % NW) * yps + t / NW;
+      const int os = z ? 1 : L;
+      PWK_SFOR(N, j, out[j * os] = x[OutSlot<N, j>::value]);
     };
-    // ss: shifts of the inputs (fixed point), at ss[j sstride]; so: where the line's own goes
-    auto forward_line = [&](const VA* in, int stride, const unsigned char* ss, int sstride, unsigned char* so, VA* pos,
-                            VA* neg, int ostride) {
+    auto forward_line = [&](bool z, int t, int l0) {
       VA x[N];
-      PWK_SFOR(N, j, x[j] = in[j * stride]);
-      *so = (unsigned char)fx_align<N>(x, ss, sstride);
+      const int srow = z ? stick_row(t) : 0;
+      VA* zp = z ? Z + srow * zs : Z + l0 + t / NW;
+      const VA* in = z ? zp : Yc + (size_t)(t % NW) * yps + t / NW;
+      const int is = z ? 1 : L;
+      PWK_SFOR(N, j, x[j] = in[j * is]);
+      const int sh = fx_align<N>(x, z ? sy + sz[srow] * N : sxc + t / NW, is);
+      (z ? sz + srow : sy + t % NW * N + l0 + t / NW)[0] = (unsigned char)sh;
       LineFFT<A, N, -1>::run(x);
       PWK_SFOR(N, j, {
         if constexpr (Wn::in(j)) {
-          if constexpr (j <= W) pos[j * ostride] = x[OutSlot<N, j>::value];
-          else neg[(j - N) * ostride] = x[OutSlot<N, j>::value];
+          const int row = z ? 0 : window_row(t % NW, Wn::idx(j));
+          if (!LIST || z || row != nz) zp[z ? j : row * zs] = x[OutSlot<N, j>::value];
         }
       });
     };
     auto x_line = [&](int t, int l0, int lc) {
       const int l2 = t / lc, c = t - l2 * lc;
       VA x[N], y[N];
-      U* yl = Yc + (size_t)l2 * L + c;
+      VA* yl = Yc + (size_t)l2 * L + c;
       PWK_SFOR(N, i, x[i] = Wn::in(i) ? yl[(size_t)Wn::idx(i) * yps] : VA{A(0), A(0)});
       LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
       sxc[l2 * L + c] = (unsigned char)fx_v_product<N>(x, static_cast<const int2*>(a.V) + ((size_t)l2 * N + l0 + c) * N, y);
@@ -233,19 +264,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
       const int lc = first || last ? 0 : min(L, N - l0);
       if (!last) {
         const int n = first ? ns : NW * lc, step = first ? nth : step0;
-        for (int t = first ? tid : lane0; t < n; t += step) {
-          const VA *pos, *neg;
-          VA* out;
-          if (first) {
-            out = Z + rows[t] * zs;
-            pos = out;
-            neg = out + N;
-          } else {
-            pos = neg = y_square(t, l0);
-            out = y_chunk(t);
-          }
-          inverse_line(pos, neg, first ? 1 : zs, out, first ? 1 : L);
-        }
+        for (int t = first ? tid : lane0; t < n; t += step) inverse_line(first, t, l0);
         if (first) {
           __syncthreads();
           l0 = warp * L;
@@ -257,26 +276,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
         sync_pass();
       }
       const int n = last ? ns : NW * lc, step = last ? nth : step0;
-      for (int t = last ? tid : lane0; t < n; t += step) {
-        const VA* in;
-        VA *pos, *neg;
-        const unsigned char* ss;
-        unsigned char* so;
-        if (last) {
-          const int row = rows[t];
-          VA* zr = Z + row * zs;
-          in = pos = zr;
-          neg = zr + N;
-          ss = sy + row / NW * N;
-          so = sz + row;
-        } else {
-          in = y_chunk(t);
-          pos = neg = y_square(t, l0);
-          ss = sxc + t / NW;
-          so = sy + t % NW * N + l0 + t / NW;
-        }
-        forward_line(in, last ? 1 : L, ss, last ? 1 : L, so, pos, neg, last ? 1 : zs);
-      }
+      for (int t = last ? tid : lane0; t < n; t += step) forward_line(last, t, l0);
       if (last) break;
       l0 += nw * L;
       if (l0 >= N) __syncthreads();

@@ -106,6 +106,7 @@ size_t fused_smem_bytes(int N, int elem_bytes, int nstick_max, int P, int L, int
 // x-pass addresses are consecutive in t: the 16 eight-byte accesses of a half-warp fall on 32
 // different banks in both passes.  zs = u^2 (mod 16) is odd, so the z pass (one stick row per
 // thread) stays conflict-free for consecutive sticks as well.
+// With lists the sticks of one m2 and consecutive m1 lie in consecutive rows: an odd zs is enough.
 void window_strides(int N, int L, int* zs, int* yps) {
   const int W = N / 4, NW = 2 * W + 1;
   int u = 1;
@@ -113,7 +114,7 @@ void window_strides(int N, int L, int* zs, int* yps) {
   const int z_res = (u * u) % 16;
   int z = N;
   while (z % 16 != z_res) ++z;
-  *zs = z;
+  *zs = window_lists(N) ? N | 1 : z;
   int y = N * L;
   while (y % 16 != u) ++y;
   *yps = y;
@@ -123,9 +124,10 @@ size_t window_smem_bytes(int N, int elem_bytes, int L, int nstick_max, int copie
   const int W = N / 4, NW = 2 * W + 1;
   int zs, yps;
   window_strides(N, L, &zs, &yps);
-  size_t elems = (size_t)NW * NW * zs + (size_t)copies * NW * yps;
-  const size_t shifts = elem_bytes == 16 ? (size_t)copies * N * L + (size_t)NW * N + 16 * (size_t)window_shift_elems(NW) : 0;
-  return elems * elem_bytes + (size_t)nstick_max * sizeof(short) + shifts + 16;
+  const size_t nrows = window_lists(N) ? nstick_max + 1 : NW * NW, ntab = window_lists(N) ? NW * NW : nstick_max;
+  size_t elems = nrows * zs + (size_t)copies * NW * yps;
+  const size_t shifts = elem_bytes == 16 ? (size_t)copies * N * L + (size_t)NW * N + 16 * (size_t)window_shift_elems((int)nrows) : 0;
+  return elems * elem_bytes + ntab * sizeof(short) + shifts + 16;
 }
 
 // ---------------------------------------------------------------- setup kernels
@@ -325,7 +327,8 @@ int build_sphere_map(pwk_plan* p, SphereMap& sm, int nk, const int* npw_in, int 
 }
 
 // Tables of the window-specialised kernel: every Miller index of the plan within
-// |m_i| <= W = N/4; the sticks of a k live at rows (m1+W)(2W+1) + (m2+W) of a dense square.
+// |m_i| <= W = N/4; the sticks of a k live at rows (m1+W)(2W+1) + (m2+W) of a dense square, or
+// (window_lists) one row after another with a table.
 int build_window_tables(pwk_plan* p) {
   const int N = p->N, W = N / 4, NW = 2 * W + 1, nk = p->nk, np = p->npw_max;
   for (size_t i = 0; i < p->h_miller.size(); ++i) {
@@ -333,20 +336,29 @@ int build_window_tables(pwk_plan* p) {
     if (g < p->h_npw[k] && std::abs(p->h_miller[i]) > W) return PWK_OK;   // not eligible
   }
   const int nsm = p->self.nstick_max;
+  const bool lists = window_lists(N);
+  const size_t ntab = lists ? (size_t)NW * NW : (size_t)nsm;
   std::vector<int> gm((size_t)nk * np, 0);
-  std::vector<short> rows((size_t)nk * nsm, (short)0);
+  std::vector<short> rows((size_t)nk * ntab, (short)(lists ? -1 : 0));
   for (int k = 0; k < nk; ++k) {
-    std::vector<char> seen((size_t)NW * NW, 0);
-    int c = 0;
-    for (int g = 0; g < p->h_npw[k]; ++g) {
+    std::vector<short> row((size_t)NW * NW, (short)-1);   // row of window cell (m2, m1), -1: no stick
+    auto cell = [&](int g) {
       const int* m = &p->h_miller[((size_t)k * np + g) * 3];
-      const int row = (m[0] + W) * NW + (m[1] + W);
-      gm[(size_t)k * np + g] = (row << 8) | (((m[2] % N) + N) % N);
-      if (!seen[row]) {
-        seen[row] = 1;
-        if (c >= nsm) return PWK_OK;   // cannot happen: same stick count as the self map
-        rows[(size_t)k * nsm + c++] = (short)row;
-      }
+      return (m[1] + W) * NW + (m[0] + W);
+    };
+    for (int g = 0; g < p->h_npw[k]; ++g) row[cell(g)] = 0;
+    int c = 0;
+    for (int i = 0; i < NW * NW; ++i) {
+      if (row[i] < 0) continue;
+      if (c >= nsm) return PWK_OK;   // cannot happen: same sticks as the self map
+      row[i] = (short)(lists ? c : (i % NW) * NW + i / NW);
+      if (!lists) rows[(size_t)k * nsm + c] = row[i];
+      ++c;
+    }
+    if (lists) std::copy(row.begin(), row.end(), rows.begin() + (size_t)k * ntab);
+    for (int g = 0; g < p->h_npw[k]; ++g) {
+      const int m3 = p->h_miller[((size_t)k * np + g) * 3 + 2];
+      gm[(size_t)k * np + g] = (row[cell(g)] << 8) | (((m3 % N) + N) % N);
     }
   }
   int rc;
@@ -394,10 +406,11 @@ static size_t fused_layout(const pwk_plan* p, int precision, const LaunchShape& 
   size_t R = r16(s.smem);
   size_t loc = 0;
   if (s.kind >= 1) {
-    const int N = p->N, NW = 2 * (N / 4) + 1;
+    const int N = p->N;
     int zs = 0, yps = 0;
     window_strides(N, s.L, &zs, &yps);
-    const size_t zb = r16((size_t)NW * NW * zs * V) + (V == 16 ? 16 * (size_t)window_shift_elems(NW) : 0);
+    const int NW = 2 * (N / 4) + 1, nrows = window_lists(N) ? p->self.nstick_max + 1 : NW * NW;
+    const size_t zb = r16((size_t)nrows * zs * V) + (V == 16 ? 16 * (size_t)window_shift_elems(nrows) : 0);
     const size_t lc = r16(2 * (size_t)p->npw_max * V);
     const size_t bb = r16((size_t)p->nkb * p->npw_max * V);
     R = std::max(R, std::max(bb, zb) + lc);

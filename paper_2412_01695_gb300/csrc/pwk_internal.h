@@ -103,8 +103,10 @@ struct pwk_plan {
   pwk::SphereMap self;
   // window-specialised kernel tables (|m_i| <= (N-1)/4 on every sphere of the plan)
   bool window_ok = false;
-  int* d_wgmap = nullptr;        // [nk][npw_max] (row << 8) | (m3 mod N), row = (m1+W)(2W+1)+(m2+W)
-  short* d_wrows = nullptr;      // [nk][nstick_max] rows of the real sticks
+  int* d_wgmap = nullptr;        // [nk][npw_max] (row << 8) | (m3 mod N)
+  short* d_wrows = nullptr;      // [nk][nstick_max] rows of the sticks, row = (m1+W)(2W+1)+(m2+W);
+                                 // window_lists: [nk][2W+1 (m2)][2W+1 (m1)] row or -1, rows
+                                 // numbered in the order of (m2, m1)
   pwk::SphereMap xfer;           // from xfer_src's spheres to this plan's (DFPT rhs)
   const pwk_plan* xfer_src = nullptr;
   pwk::LaunchShape shape[3];     // per precision
@@ -233,8 +235,13 @@ int launch_window_f32c128(int N, const FusedArgs& a, int nblocks, const LaunchSh
                           cudaStream_t st);
 // copies: plane buffers (1 for a CTA-wide chunk, the warp count for per-warp planes)
 size_t window_smem_bytes(int N, int elem_bytes, int L, int nstick_max, int copies);
-// 16-byte elements that hold the shifts of the (2W+1)^2 z lines (FP64 window kernel)
-__host__ __device__ constexpr int window_shift_elems(int nw) { return (nw * nw + 15) / 16; }
+// Whether the window kernel keeps the sticks of a grid as a list with a table instead of a dense
+// square.  At N = 36 (cell of 4 atoms, 8 of 9 window indices used) the list is half the square and
+// two CTAs fit an SM: H|psi> of 343 k x 40 bands in FP32 2.94 -> 2.54 ms.  At N = 24 the square
+// already leaves room for four CTAs and the table only costs: 397 -> 408 us (512 k x 20 bands).
+__host__ __device__ constexpr bool window_lists(int N) { return N >= 30; }
+// 16-byte elements that hold the shifts of n z lines (FP64 window kernel)
+__host__ __device__ constexpr int window_shift_elems(int n) { return (n + 15) / 16; }
 // strides of the window kernel's shared buffers for chunk L (bank-conflict-free y/x passes)
 void window_strides(int N, int L, int* zs, int* yps);
 

@@ -141,3 +141,46 @@ def test_fields(field):
             assert np.all(np.isnan(y[k, :, :prob.npw[k]].real))
         return
     check(prob, x, y)
+
+
+SC = synth.sc_lattice(7.5)
+SITES = 7.5 * np.array([[0, 0, 0], [0, 0.5, 0.5], [0.5, 0, 0.5], [0.5, 0.5, 0]])
+
+
+@pytest.mark.parametrize("N,nat,lset", [(12, 1, (0,)), (16, 4, (0, 1, 2)), (15, 1, (0, 1)), (32, 1, (0, 1)),
+                                        (20, 2, (0, 1, 2))])
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("spread", [0, 150])
+def test_projector_terms_in_limbs(N, nat, lset, kind, spread):
+    """The integer projector sums inside the FP64 kernel: one projector, more than the 31 an
+    accumulator holds in the add-back (36), more plane waves than it holds in a lane (1500 > 31 *
+    32), and projectors of very different size (2^-spread to 2^spread, the coefficients scaled
+    back).  H and S against long double; the bar is that of the H tests (the limbs hold 57 bits of
+    the largest component, the left-out products 2^-56 of the largest product)."""
+    torch = torch_cuda()
+    from paper_2412_01695_gb300 import pwk
+    ecut = ((N // 4 + 0.4) * 2 * np.pi / 7.5) ** 2 * 0.9
+    k = synth.mp_grid(synth.reciprocal_rows(SC), (1, 1, 1)) + 0.05
+    prob = synth.build_problem(SC, SITES[:nat], lset, N, ecut, k, 4, 1, with_psi=False)
+    q = synth.random_q(np.random.default_rng(2), nat, lset)
+    s = 2.0 ** np.linspace(-spread, spread, prob.nkb).round() if prob.nkb > 1 else np.ones(1)
+    prob.beta = np.ascontiguousarray(prob.beta * s[None, :, None])
+    prob.D = prob.D / np.outer(s, s)
+    q = q / np.outer(s, s)
+    x = vectors(prob)
+    plan = pwk.plan_from_problem(prob)
+    plan.set_overlap(q)
+    plan.set_launch_shape(pwk.PWK_FP64, kind, 128, max(1, N // 8))
+    plan.set_projector_path(3)
+    assert plan.projector_fused(pwk.PWK_FP64)
+    d = torch.from_numpy(x).cuda()
+    h, sp = torch.full_like(d, complex(np.nan, np.nan)), torch.full_like(d, complex(np.nan, np.nan))
+    pwk.hspsi_batched(plan, pwk.PWK_FP64, d, h, sp, x.shape[1])
+    torch.cuda.synchronize()
+    plan.close()
+    check(prob, x, h.cpu().numpy())
+    n = int(prob.npw[0])
+    b = prob.beta[0][:, :n].astype(np.clongdouble)
+    for v, got in zip(x[0], sp.cpu().numpy()[0]):
+        ref = v[:n] + ((v[:n].astype(np.clongdouble) @ b.conj().T) @ q) @ b
+        assert np.linalg.norm((got[:n] - ref).astype(complex)) <= 5e-16 * max(np.linalg.norm(ref.astype(complex)), 1e-300)
