@@ -19,6 +19,7 @@
 #include "fft_line.cuh"
 #include "fixed_block.cuh"
 #include "fused_kernel.cuh"
+#include "nl_fused.cuh"
 #include "pwk_internal.h"
 #include "solvers.h"
 
@@ -42,6 +43,12 @@ struct DrhoArgs {
   const short* sid = nullptr;
   int nstick_max = 0, m1lo = 0, P = 0, L = 0, zs = 0;
 };
+
+// v 2^e for an integer value v (0, or 1 <= |v| < 2^62) and fx_plain_scale(e): on the exponent field
+__device__ __forceinline__ double times_pow2(double v, int e) {
+  const int h = __double2hiint(v);
+  return h == 0 ? v : __hiloint2double(h + (e << 20), __double2loint(v));
+}
 
 // CTAs per SM the registers allow for: an FP64 line of N <= 20 fits 128 registers
 template <typename T, int N>
@@ -78,7 +85,7 @@ __global__ void __launch_bounds__(256, drho_ctas<T, N>()) drho_kernel(DrhoArgs a
     const int k = pr / a.nocc, v = pr - k * a.nocc;
     const int ns = a.nstick[k];
     const int nka = a.npwk[k], nkb = a.npwq[k];
-    double wk = 4.0 * a.w[k];
+    const double wk = 4.0 * a.w[k];
     const double2* pu = static_cast<const double2*>(a.uk) + ((size_t)k * a.nocc + v) * a.npw_k;
     const double2* pd = a.du + ((size_t)k * a.nocc + v) * a.npw_kq;
     __syncthreads();   // the previous pair is done with the buffers
@@ -88,20 +95,24 @@ __global__ void __launch_bounds__(256, drho_ctas<T, N>()) drho_kernel(DrhoArgs a
       for (int i = tid; i < P * N; i += nth) sid[i] = sk[i];
     }
     FxScale su{1.0, 0.0, 0, false, 0}, sd = su;
-    int shift_u = 0;   // exponent taken into u at the product (0 unless the pair's is extreme)
+    int eu = 0, ed = 0;          // powers of two that u and du take at the product
+    bool plain = true;
     if constexpr (FX) {
       FxScratch* scratch = fx_scratch_at(reinterpret_cast<unsigned char*>(sid + P * N));
       su = fx_block_scale(pu, nka, scratch);
       __syncthreads();
       sd = fx_block_scale(pd, nkb, scratch);
-      const int e = -su.exp - sd.exp;
-      if (fx_plain_scale(e)) {
-        wk = fx_factor(wk, e);
-      } else {
-        wk = ldexp(wk, -sd.exp);
-        shift_u = -su.exp;
+      // the weight goes into the scale of du (its mantissa, in [1/2, 1)) and of u (a power of two),
+      // so that a grid point takes two multiply-adds per component
+      int we = 0;
+      sd.in *= frexp(wk, &we);
+      if (su.bad || sd.bad || !isfinite(wk)) sd.in = 0.0;
+      eu = we - su.exp - sd.exp;
+      plain = fx_plain_scale(eu) && !su.bad && !sd.bad && isfinite(wk);
+      if (!plain) {
+        eu = -su.exp;
+        ed = su.bad || sd.bad || !isfinite(wk) ? kFxBadField : we - sd.exp;
       }
-      if (su.bad || sd.bad) wk = __longlong_as_double(0x7ff8000000000000LL);
     }
     __syncthreads();
     {
@@ -163,20 +174,28 @@ __global__ void __launch_bounds__(256, drho_ctas<T, N>()) drho_kernel(DrhoArgs a
           if (f == 0) {
             PWK_SFOR(N, l1, {
               V z = drho_value<V>(x[OutSlot<N, l1>::value]);
-              if constexpr (FX) {
-                if (shift_u != 0) z = V{ldexp(z.x, shift_u), ldexp(z.y, shift_u)};   // uniform
-              }
+              if constexpr (FX) z = plain ? V{times_pow2(z.x, eu), times_pow2(z.y, eu)} : V{ldexp(z.x, eu), ldexp(z.y, eu)};
               xa[(size_t)l1 * N * L] = z;
             });
           } else {
             double2* ag = acc + (size_t)l2 * N + l0 + c;
             PWK_SFOR(N, l1, {
-              const V ua = xa[(size_t)l1 * N * L], ub = drho_value<V>(x[OutSlot<N, l1>::value]);
-              const double re = (double)ua.x * ub.x + (double)ua.y * ub.y;   // conj(u) du
-              const double im = (double)ua.x * ub.y - (double)ua.y * ub.x;
-              double2& d = ag[(size_t)l1 * N * N];
-              d.x += wk * re;
-              d.y += wk * im;
+              const V ua = xa[(size_t)l1 * N * L];
+              V ub = drho_value<V>(x[OutSlot<N, l1>::value]);
+              double2& d = ag[(size_t)l1 * N * N];   // += conj(u) du (times the weight, FP64: in the scales)
+              if constexpr (FX) {
+                if (!plain) {   // uniform
+                  const double bad = __longlong_as_double(0x7ff8000000000000LL);
+                  ub = ed == kFxBadField ? V{bad, bad} : V{ldexp(ub.x, ed), ldexp(ub.y, ed)};
+                }
+                d.x = fma(ua.x, ub.x, fma(ua.y, ub.y, d.x));
+                d.y = fma(ua.x, ub.y, fma(-ua.y, ub.x, d.y));
+              } else {
+                const double re = (double)ua.x * ub.x + (double)ua.y * ub.y;
+                const double im = (double)ua.x * ub.y - (double)ua.y * ub.x;
+                d.x += wk * re;
+                d.y += wk * im;
+              }
             });
           }
         }
@@ -210,45 +229,66 @@ __global__ void __launch_bounds__(256) drho_reduce_kernel(int nr, int nparts, co
   out[l] = make_double2(sx, sy);
 }
 
-// P_c du = du - sum_v u_v <su_v|du> (su = S u, or u when S = 1), one CTA per (k, nu)
+// Exponent of a vector of np complex numbers by one warp: every |component| < 2^exponent
+// (kFxBadField: one is not finite)
+__device__ __forceinline__ int warp_exponent(const double2* v, int np) {
+  unsigned h = 0;
+  for (int g = threadIdx.x & 31; g < np; g += 32) h = max(h, max(fx_abs_hi(v[g].x), fx_abs_hi(v[g].y)));
+  h = __reduce_max_sync(0xffffffffu, h);
+  return (h >> 20) == 0x7ff ? kFxBadField : (int)(h >> 20) - 1022;
+}
+
+// P_c du = du - sum_v u_v <su_v|du> (su = S u, or u when S = 1), one CTA per (k, nu).  The two
+// contractions are the projector sums of nl_fused.cuh with the valence states as projectors, on
+// the integer pipe: with FP64 multiply-adds they held that pipe (85 % busy) for 113 us on 768 pairs
+// of 12 valence states.
 __global__ void __launch_bounds__(256) conduction_kernel(int nocc, int np, const int* npw,
                                                          const double2* u, const double2* su,
                                                          const double2* du, double2* out) {
   const int k = blockIdx.x / nocc;
   const int npk = npw[k];
-  __shared__ double2 mu[64];
+  __shared__ double2 buf[2 * 64];   // the second half: <su_v|du>, then its limbs
+  __shared__ int eu[64], es[64], ex[2], ed;
   const double2* D = du + (size_t)blockIdx.x * np;
   const double2* U = u + (size_t)k * nocc * np;
   const double2* SU = su + (size_t)k * nocc * np;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int v = warp; v < nocc; v += nw) {
-    double sx = 0, sy = 0;
-    const double2* s = SU + (size_t)v * np;
-    for (int g = lane; g < npk; g += 32) {
-      const double2 a = s[g], b = D[g];
-      sx += a.x * b.x + a.y * b.y;
-      sy += a.x * b.y - a.y * b.x;
+  for (int v = warp; v <= nocc; v += nw) {
+    const int e = warp_exponent(v < nocc ? U + (size_t)v * np : D, npk);
+    const int e2 = v < nocc && su != u ? warp_exponent(SU + (size_t)v * np, npk) : e;
+    if (lane == 0) {
+      if (v < nocc) {
+        eu[v] = e;
+        es[v] = e2;
+      } else {
+        ed = e;
+      }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      sx += __shfl_xor_sync(0xffffffffu, sx, o);
-      sy += __shfl_xor_sync(0xffffffffu, sy, o);
-    }
-    if (lane == 0) mu[v] = make_double2(sx, sy);
   }
   __syncthreads();
   double2* O = out + (size_t)blockIdx.x * np;
+  const int ce = ed;
+  if (ce == kFxBadField) {   // uniform: a component of du is not finite
+    for (int g = threadIdx.x; g < np; g += blockDim.x) O[g] = g < npk ? make_double2(nan(""), nan("")) : make_double2(0.0, 0.0);
+    return;
+  }
+  auto limbs = [&](const double2* base, const int* e, int v, int g) {
+    return nl_limbs(base[(size_t)v * np + g], e[v] == kFxBadField ? 0 : e[v]);
+  };
+  nl_fx_project(nocc, npk, es, ce, [&](int v, int g) { return limbs(SU, es, v, g); },
+                [&](int g) { return nl_limbs(D[g], ce); }, buf + nocc);
+  __syncthreads();
+  nl_fx_coef(nocc, false, eu, buf, ex);
+  __syncthreads();
+  const int4* mu = reinterpret_cast<const int4*>(buf + nocc);
   for (int g = threadIdx.x; g < np; g += blockDim.x) {
     if (g >= npk) {
       O[g] = make_double2(0.0, 0.0);
       continue;
     }
-    double2 r = D[g];
-    for (int v = 0; v < nocc; ++v) {
-      const double2 p = U[(size_t)v * np + g], m = mu[v];
-      r.x -= p.x * m.x - p.y * m.y;
-      r.y -= p.x * m.y + p.y * m.x;
-    }
-    O[g] = r;
+    double2 h, unused;
+    nl_fx_addback(nocc, g, mu, ex, false, [&](int v, int i) { return limbs(U, eu, v, i); }, h, unused);
+    O[g] = make_double2(D[g].x - h.x, D[g].y - h.y);
   }
 }
 
