@@ -770,7 +770,7 @@ extern "C" int pwk_davidson_batched(pwk_plan* p, int mode, void* psi_v, double* 
     set_nbase_kernel<<<blocks(nk), 256, 0, st>>>(nk, mask, w->nbase, nb, nullptr); note_launch();
     cudaEvent_t tr = T.mark();
     r = launch_rr(nk, MB, nb, w->nbase, mask, w->Hr, w->Sr, w->W, w->ev, w->eps_new, w->status, st,
-                  w->drop, rr_flops);
+                  w->drop, rr_flops, count);
     T.close(1, tr);
     return r;
   };
@@ -907,7 +907,7 @@ extern "C" int pwk_davidson_batched(pwk_plan* p, int mode, void* psi_v, double* 
       KCHECK("davidson gram");
       cudaEvent_t tr = T.mark();
       if ((rc = launch_rr(nk, MB, nb, w->nbase, w->iterk, w->Hr, w->Sr, w->W, w->ev, w->eps_new,
-                          w->status, st, w->drop, rr_flops)))
+                          w->status, st, w->drop, rr_flops, hc[6])))
         return rc;
       T.close(1, tr);
       trace_reduced(w, it);

@@ -743,14 +743,16 @@ __global__ void __launch_bounds__(512, 2) rr_kernel(int nk, int ld, int nb, cons
 }
 
 // Threads per problem: 512 where a CTA has an SM to itself and enough rows to fill them, 256 for
-// small problems and where several CTAs share an SM (n = 80, 20 vectors, 512 problems: 7.4 ms
-// with 256, 8.6 with 512; 128 problems: 2.7 with 512).
-static int rr_threads(int nk, int ld) { return ld > 40 && nk <= 304 ? 512 : 256; }
+// small problems and where several CTAs share an SM (n = 80, 20 vectors, 512 problems: 7.5 ms
+// with 256, 8.6 with 512; 128 problems: 2.64 with 512).  The Davidson passes the number of k-points
+// still active, so the tail of a large solve takes the wide form (512 k x 20 bands: eigensolves 406
+// -> 396 ms of the solve).
+static int rr_threads(int nactive, int ld) { return ld > 40 && nactive <= 304 ? 512 : 256; }
 
 int launch_rr(int nk, int ld, int nb, const int* nbase, const int* active, const double2* Hr,
               const double2* Sr, double2* W, double2* ev, double* eps, int* status,
-              cudaStream_t st, unsigned char* drop_out, double* flops) {
-  rr_kernel<<<nk, rr_threads(nk, ld), 0, st>>>(nk, ld, nb, nbase, active, Hr, Sr, W, ev, eps, status, drop_out, flops); note_launch();
+              cudaStream_t st, unsigned char* drop_out, double* flops, int nactive) {
+  rr_kernel<<<nk, rr_threads(nactive < 0 ? nk : nactive, ld), 0, st>>>(nk, ld, nb, nbase, active, Hr, Sr, W, ev, eps, status, drop_out, flops); note_launch();
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? PWK_OK : cuda_fail(e, "rr_kernel");
 }

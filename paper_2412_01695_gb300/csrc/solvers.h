@@ -16,9 +16,11 @@ void destroy_cg_work(pwk_plan* p);
 // drop_out (optional, [nk][ld]): 1 for each basis vector left out as numerically dependent
 // flops (optional, device): the algorithmic FP64 operation count of every problem solved is
 // added to it
+// nactive: how many of the nk problems are active where the caller knows (-1: nk); it only
+// chooses the threads per problem
 int launch_rr(int nk, int ld, int nb, const int* nbase, const int* active, const double2* Hr,
               const double2* Sr, double2* W, double2* ev, double* eps, int* status,
-              cudaStream_t st, unsigned char* drop_out = nullptr, double* flops = nullptr);
+              cudaStream_t st, unsigned char* drop_out = nullptr, double* flops = nullptr, int nactive = -1);
 
 // Device time of the phases of a solver call (pwk_plan_set_solver_timing): CUDA events are
 // recorded around each phase on the solver's stream and read after the stream synchronises
