@@ -22,19 +22,13 @@
 
 namespace pwk {
 
-// projectors per warp group in the prologue (accumulators held in registers)
-template <typename T>
-struct NlGroup {
-  static constexpr int G = sizeof(T) == 4 ? 4 : 3;
-};
-
 // Prologue, part 1: lambda of every projector into nls[0, nkb).  C(G) is read through
 // `cin`, beta(k) through `bk` ([nkb][ldb]); either may be global or shared memory.
 template <typename T, typename CV>
 __device__ __forceinline__ void nl_fused_project(const FusedArgs& a, const c2_t<T>* bk, int ldb,
                                                  const CV* cin, int np, c2_t<T>* nls) {
   using V = c2_t<T>;
-  constexpr int G = NlGroup<T>::G;
+  constexpr int G = 4;   // projectors per warp group (accumulators held in registers)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int ngroups = (a.nkb + G - 1) / G;
   for (int grp = warp; grp < ngroups; grp += nw) {
@@ -121,7 +115,7 @@ __device__ __forceinline__ void nl_fused_addback(const FusedArgs& a, const c2_t<
 
 // beta(k) ([nkb][npw_beta] contiguous) into shared memory at dst by asynchronous copies from
 // every thread of the CTA (16-byte copies when the block is 16-byte aligned and sized, else one
-// complex element per copy); returns once every copy has landed and the CTA has synchronised.
+// complex element per copy), FP32; returns once every copy has landed and the CTA has synchronised.
 template <typename T>
 __device__ __forceinline__ void nl_stage_beta(const FusedArgs& a, int k, c2_t<T>* dst) {
   using V = c2_t<T>;
@@ -134,12 +128,9 @@ __device__ __forceinline__ void nl_stage_beta(const FusedArgs& a, int k, c2_t<T>
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d0 + (unsigned)i), "l"(s + i) : "memory");
   } else {
     for (size_t i = threadIdx.x; i < n; i += blockDim.x) {
-      if constexpr (sizeof(V) == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d0 + (unsigned)(i * 16)), "l"(src + i)
-                     : "memory");
-      else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d0 + (unsigned)(i * 8)), "l"(src + i)
-                     : "memory");
+      static_assert(sizeof(V) == 8, "FP32 vectors");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d0 + (unsigned)(i * 8)), "l"(src + i)
+                   : "memory");
     }
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
