@@ -65,8 +65,11 @@ __device__ __forceinline__ int plane_of_slot(int i, int m1lo) {
   return p < 0 ? p + N : (p >= N ? p - N : p);
 }
 
-// NL: the projector terms are applied as well (nl_fused.cuh: projections after the scatter
-// from the staged C, add-back in the gather, beta(k) read through L1/L2); compiled apart.
+// NL: the projector terms are applied as well (nl_fused.cuh: projections after the scatter, from
+// the staged C in FP32 and from global memory in FP64, add-back in the gather, beta(k) read
+// through L1/L2); compiled apart.
+// Threads: an FP64 line of N <= 25 fits the 168 registers of 384 threads per SM, so two CTAs of
+// 192 can share one (at 256 the compiler takes up to 255 registers and one CTA fits).
 template <typename T, typename TI, int N, bool CPLXV, bool NL>
 __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_kernel(FusedArgs a) {
   using V = c2_t<T>;
