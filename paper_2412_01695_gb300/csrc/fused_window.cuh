@@ -207,10 +207,12 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
         if constexpr (Wn::in(j)) zr[j] = x[OutSlot<N, j>::value];
       });
     }
+    __syncthreads();
   } else {
     // fixed point: one copy of the inverse and of the forward code for the z and y lines
     // (unrolled over a line it is thousands of instructions, and the instruction cache holds
-    // few): stages -1 (inverse z), a chunk's y, x, y each, N (forward z).
+    // few): stages inverse z, the chunks' y, x, y, forward z, with one block barrier that ends
+    // each stage for every warp, also one without a chunk of its own.
     // z: the line is stick t; y: plane t % NW of column l0 + t / NW, its window elements in the
     // rows of the table.
     unsigned char* sxc = sx + (size_t)warp * N * L;
@@ -259,31 +261,28 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
         if constexpr (Wn::in(i)) yl[(size_t)Wn::idx(i) * yps] = y[OutSlot<N, i>::value];
       });
     };
-    for (int l0 = -1;;) {
-      const bool first = l0 < 0, last = l0 >= N;
-      const int lc = first || last ? 0 : min(L, N - l0);
-      if (!last) {
-        const int n = first ? ns : NW * lc, step = first ? nth : step0;
-        for (int t = first ? tid : lane0; t < n; t += step) inverse_line(first, t, l0);
-        if (first) {
-          __syncthreads();
-          l0 = warp * L;
-          if (l0 >= N) __syncthreads();   // a warp without chunks: the barrier before the last stage
-          continue;
+#pragma unroll 1
+    for (int stage = 0; stage < 3; ++stage) {   // uniform: every warp meets the barrier below three times
+      const bool first = stage == 0, last = stage == 2;
+      // the chunks of stage 1; the z stages take the body once
+#pragma unroll 1
+      for (int l0 = stage == 1 ? warp * L : 0; l0 < (stage == 1 ? N : 1); l0 += nw * L) {
+        const int lc = min(L, N - l0);
+        const int n = stage == 1 ? NW * lc : ns, t0 = stage == 1 ? lane0 : tid, step = stage == 1 ? step0 : nth;
+        if (!last)
+          for (int t = t0; t < n; t += step) inverse_line(first, t, l0);
+        if (stage == 1) {
+          sync_pass();
+          for (int t = lane0; t < N * lc; t += step0) x_line(t, l0, lc);
+          sync_pass();
         }
-        sync_pass();
-        for (int t = lane0; t < N * lc; t += step0) x_line(t, l0, lc);
-        sync_pass();
+        if (!first)
+          for (int t = t0; t < n; t += step) forward_line(last, t, l0);
+        if (stage == 1 && l0 + nw * L < N) sync_pass();   // another chunk reuses the planes
       }
-      const int n = last ? ns : NW * lc, step = last ? nth : step0;
-      for (int t = last ? tid : lane0; t < n; t += step) forward_line(last, t, l0);
-      if (last) break;
-      l0 += nw * L;
-      if (l0 >= N) __syncthreads();
-      else sync_pass();
+      __syncthreads();
     }
   }
-  __syncthreads();
 
   // ---- 5: gather with 1/N_r; kinetic term
   const int vexp = a.vexp == kFxBadField ? 0 : a.vexp;

@@ -9,7 +9,7 @@ size, zero and non-finite vectors, V constant, V = 0, V large and tiny."""
 import numpy as np
 import pytest
 
-from paper_2412_01695_gb300 import synth
+from paper_2412_01695_gb300 import pwk, synth
 
 from gpu_util import torch_cuda
 
@@ -92,6 +92,25 @@ def test_every_kind_at_every_radix(N, kind):
     prob = problem(N)
     x = vectors(prob)
     check(prob, x, apply(prob, x, (kind, 128, 1 if kind == 2 else max(1, N // 8))))
+
+
+@pytest.mark.parametrize("N", [12, 15, 32])
+def test_warps_without_planes(N):
+    """Kind 2 with more warps than the grid has chunks (N = 12, two planes per warp: six of eight
+    warps), with a chunk each, and with several: every warp meets the same block barriers, and
+    the bits are those of the CTA-wide kind."""
+    prob = problem(N)
+    x = vectors(prob)
+    first = apply(prob, x, (1, 128, max(1, N // 4)))
+    check(prob, x, first)
+    for threads in (96, 128, 192, 256):
+        for L in (1, 2):
+            try:
+                y = apply(prob, x, (2, threads, L))
+            except pwk.PwkError as e:
+                assert e.code == -2   # the planes of so many warps do not fit in shared memory
+                continue
+            assert np.array_equal(y, first), (threads, L)
 
 
 @pytest.mark.parametrize("exponent", [-1060, -900, -300, 300, 900])
