@@ -86,6 +86,9 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
   unsigned char* sy = sx + (size_t)ycopies * N * L;
   auto stick_row = [&](int s) { return LIST ? s : (int)tab[s]; };
   auto window_row = [&](int p, int i) { return LIST ? (int)tab[i * NW + p] : p * NW + i; };   // plane p, m2 index i
+  // the same in two parts: on the square the rows of a plane lie at fixed steps from its first
+  auto plane_at = [&](int p) { return LIST ? Z : Z + (size_t)p * NW * zs; };
+  auto plane_row = [&](int p, int i) { return LIST ? (int)tab[i * NW + p] : i; };
 
   const VI* pin = static_cast<const VI*>(a.in) + ((size_t)k * a.nvec_in + vin) * a.npw_in_max;
   VI* pout = static_cast<VI*>(a.out) + ((size_t)k * a.nvec_out + vout) * a.npw_out_max;
@@ -152,9 +155,9 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
       for (int t = lane0; t < NW * lc; t += step0) {
         const int c = t / NW, p = t - c * NW;   // plane fastest: see window_strides
         VA x[N];
-        const VA* zp = Z + l0 + c;
+        const VA* zp = plane_at(p) + l0 + c;
         PWK_SFOR(N, j, {
-          if constexpr (Wn::in(j)) x[j] = zp[window_row(p, Wn::idx(j)) * zs];
+          if constexpr (Wn::in(j)) x[j] = zp[plane_row(p, Wn::idx(j)) * zs];
           else x[j] = VA{A(0), A(0)};
         });
         LineFFTZ<A, N, +1, OutOfWin<N, W>>::run(x);
@@ -187,10 +190,10 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
         const VA* yp = Yc + (size_t)p * yps + c;
         PWK_SFOR(N, l2, x[l2] = yp[l2 * L]);
         LineFFT<A, N, -1>::run(x);
-        VA* zp = Z + l0 + c;
+        VA* zp = plane_at(p) + l0 + c;
         PWK_SFOR(N, j, {
           if constexpr (Wn::in(j)) {
-            const int row = window_row(p, Wn::idx(j));
+            const int row = plane_row(p, Wn::idx(j));
             if (!LIST || row != nz) zp[row * zs] = x[OutSlot<N, j>::value];
           }
         });
@@ -287,25 +290,23 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
   // ---- 5: gather with 1/N_r; kinetic term
   const int vexp = a.vexp == kFxBadField ? 0 : a.vexp;
   const double scd = FX && (scale.bad || a.vexp == kFxBadField) ? __longlong_as_double(0x7ff8000000000000LL) : a.scale;
-  auto local = [&](int m) -> V {   // the local term of the basis vector at packed place m
+  const T sc = T(scd);
+  // the local term of the basis vector at packed place m, with the kinetic term t2 c
+  auto local = [&](int m, T t2, VI c) -> V {
     const VA z = Z[(m >> 8) * zs + (m & 255)];
     if constexpr (FX) {
       const int e = sz[m >> 8] + vexp - scale.exp;
       const double f = fx_factor(scd, e);
-      return V{fx_scaled(z.x, f, e), fx_scaled(z.y, f, e)};
+      return V{fx_scaled(z.x, f, e) + t2 * c.x, fx_scaled(z.y, f, e) + t2 * c.y};
     } else {
-      const T sc = T(scd);
-      return V{z.x * sc, z.y * sc};
+      return V{z.x * sc + t2 * T(c.x), z.y * sc + t2 * T(c.y)};
     }
   };
   if (!NL || a.nkb == 0) {
     const int* gout = a.gout + (size_t)k * a.npw_out_max;
     const double* g2k = a.g2 + (size_t)k * a.npw_out_max;
     for (int g = tid; g < np; g += nth) {
-      const V z = local(gout[g]);
-      const T t2 = T(g2k[g]);
-      const VI cv = pin[g];
-      V acc = V{z.x + t2 * T(cv.x), z.y + t2 * T(cv.y)};
+      const V acc = local(gout[g], T(g2k[g]), pin[g]);
       pout[g] = VI{TI(acc.x), TI(acc.y)};
     }
     for (int g = np + tid; g < a.npw_out_max; g += nth) pout[g] = VI{TI(0), TI(0)};
@@ -319,10 +320,8 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     V* Cs = LOC + a.npw_out_max;                             // [npw_out_max] C in T (FP64: limbs)
     V* nls = reinterpret_cast<V*>(smem_raw + a.nl_off);
     for (int g = tid; g < np; g += nth) {
-      const V z = local(gout[g]);
-      const T t2 = T(g2k[g]);
       const VI cv = pin[g];
-      LOC[g] = V{z.x + t2 * T(cv.x), z.y + t2 * T(cv.y)};
+      LOC[g] = local(gout[g], T(g2k[g]), cv);
       if constexpr (FX) reinterpret_cast<int4*>(Cs)[g] = nl_limbs(cv, scale.top);
       else Cs[g] = V{T(cv.x), T(cv.y)};
     }
