@@ -36,7 +36,7 @@ struct FxScale {
   double pre, in;   // the integers hold (C pre) in
   int exp;          // = C 2^exp
   bool bad;
-  int top;          // every |component of C| < 2^top
+  int top;          // every |component of C| < 2^top (bad: kFxBadField)
 };
 __device__ __forceinline__ longlong2 fx_from(const FxScale& s, double2 v) {
   if (s.pre != 1.0) v = make_double2(v.x * s.pre, v.y * s.pre);   // uniform over the block
@@ -76,7 +76,7 @@ __device__ __forceinline__ FxScale fx_block_scale(const double2* __restrict__ c,
     __syncthreads();   // hmax is read before it is reset
   }
   const int em = (int)(hm >> 20);
-  if (em == 0x7ff) return FxScale{1.0, 0.0, 0, true, 0};
+  if (em == 0x7ff) return FxScale{1.0, 0.0, 0, true, kFxBadField};
   if (em < 128) return FxScale{1.0, 0.0, 0, false, 0};   // a zero vector (pre has lifted every other one)
   // sum of the component magnitudes in units of 2^(em - 1043), each rounded up
   unsigned s0 = 0, s1 = 0;

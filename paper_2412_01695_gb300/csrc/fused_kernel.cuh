@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
   };
   if constexpr (nl) {
     if constexpr (FX)
-      nl_fx_project(a.nkb, npi, be, scale.top, load_b, [&](int g) { return nl_limbs(pin[g], scale.top); }, nls);
+      nl_fx_project(a.nkb, npi, be, scale.top, load_b, [&](int g) { return scale.bad ? int4{0, 0, 0, 0} : nl_limbs(pin[g], scale.top); }, nls);
     else
       nl_fused_project<T>(a, nl_bk, a.npw_beta, psis, npi, nls);
   }

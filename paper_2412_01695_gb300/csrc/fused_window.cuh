@@ -322,7 +322,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     for (int g = tid; g < np; g += nth) {
       const VI cv = pin[g];
       LOC[g] = local(gout[g], T(g2k[g]), cv);
-      if constexpr (FX) reinterpret_cast<int4*>(Cs)[g] = nl_limbs(cv, scale.top);
+      if constexpr (FX) reinterpret_cast<int4*>(Cs)[g] = scale.bad ? int4{0, 0, 0, 0} : nl_limbs(cv, scale.top);
       else Cs[g] = V{T(cv.x), T(cv.y)};
     }
     __syncthreads();

@@ -191,7 +191,8 @@ __device__ __forceinline__ double nl_scaled(double v, int e) {   // v 2^e
 }
 
 // Prologue, part 1 (nl_fused_project): load_b(m, g), load_c(g) give the limbs of beta_m and C
-// (C below 2^ce); bexp: exponents of the projectors of this k-point.
+// (C below 2^ce; ce = kFxBadField: C has a component that is not finite, and lambda is NaN); bexp:
+// exponents of the projectors of this k-point.
 template <typename LB, typename LC>
 __device__ __forceinline__ void nl_fx_project(int nkb, int np, const int* bexp, int ce, const LB& load_b,
                                               const LC& load_c, double2* nls) {
@@ -224,8 +225,9 @@ __device__ __forceinline__ void nl_fx_project(int nkb, int np, const int* bexp, 
       }
       if (lane == 0 && j < nc) {
         const int be = bexp[m0 + j];
-        if (be == kFxBadField) tot[j] = make_double2(nan(""), nan(""));
-        const int e = (be == kFxBadField ? 0 : be) + ce - 85;   // 2^29 / 2^114
+        const bool bad = be == kFxBadField || ce == kFxBadField;
+        if (bad) tot[j] = make_double2(nan(""), nan(""));
+        const int e = bad ? 0 : be + ce - 85;   // 2^29 / 2^114
         nls[m0 + j] = make_double2(nl_scaled(tot[j].x, e), nl_scaled(tot[j].y, e));
       }
     }

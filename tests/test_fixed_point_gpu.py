@@ -141,6 +141,31 @@ def test_a_non_finite_vector_spoils_only_itself(bad, path):
     check(prob, x, y)
 
 
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("path,kind", [(2, 1), (3, 0), (3, 1), (3, 2)])
+def test_s_of_a_non_finite_vector(bad, path, kind):
+    """One component that is not finite makes every projection NaN, so all of H C and S C, in that
+    vector alone."""
+    torch = torch_cuda()
+    prob = problem(16)
+    x = vectors(prob)
+    x[0, 2, 5] = bad
+    plan = pwk.plan_from_problem(prob)
+    plan.set_overlap(synth.random_q(np.random.default_rng(2), 1, (0, 1)))
+    plan.set_projector_path(path)
+    plan.set_launch_shape(pwk.PWK_FP64, kind, 128, 1)
+    assert plan.projector_fused(pwk.PWK_FP64) == (path == 3)
+    d = torch.from_numpy(x).cuda()
+    h, s = torch.full_like(d, 7.0), torch.full_like(d, 7.0)
+    pwk.hspsi_batched(plan, pwk.PWK_FP64, d, h, s, x.shape[1])
+    torch.cuda.synchronize()
+    plan.close()
+    n = int(prob.npw[0])
+    for out in (h.cpu().numpy()[0], s.cpu().numpy()[0]):
+        assert np.all(np.isnan(out[2, :n].real) & np.isnan(out[2, :n].imag))
+        assert np.all(np.isfinite(out[[0, 1, 3]]))
+
+
 @pytest.mark.parametrize("field", ["zero", "constant", "large", "tiny", "spike", "nan"])
 def test_fields(field):
     N = 20
