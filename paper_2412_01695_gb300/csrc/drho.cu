@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(256) conduction_kernel(int nocc, int np, const
   const int k = blockIdx.x / nocc;
   const int npk = npw[k];
   __shared__ double2 buf[2 * 64];   // the second half: <su_v|du>, then its limbs
-  __shared__ int eu[64], es[64], ex[2], ed;
+  __shared__ int eu[64], es[64], ex, ed;
   const double2* D = du + (size_t)blockIdx.x * np;
   const double2* U = u + (size_t)k * nocc * np;
   const double2* SU = su + (size_t)k * nocc * np;
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(256) conduction_kernel(int nocc, int np, const
   nl_fx_project(nocc, npk, es, ce, [&](int v, int g) { return limbs(SU, es, v, g); },
                 [&](int g) { return nl_limbs(D[g], ce); }, buf + nocc);
   __syncthreads();
-  nl_fx_coef(nocc, false, eu, buf, ex);
+  nl_fx_coef(nocc, eu, buf, &ex);
   __syncthreads();
   const int4* mu = reinterpret_cast<const int4*>(buf + nocc);
   for (int g = threadIdx.x; g < np; g += blockDim.x) {
@@ -286,8 +286,7 @@ __global__ void __launch_bounds__(256) conduction_kernel(int nocc, int np, const
       O[g] = make_double2(0.0, 0.0);
       continue;
     }
-    double2 h, unused;
-    nl_fx_addback(nocc, g, mu, ex, false, [&](int v, int i) { return limbs(U, eu, v, i); }, h, unused);
+    const double2 h = nl_fx_addback(nocc, g, mu, ex, [&](int v, int i) { return limbs(U, eu, v, i); });
     O[g] = make_double2(D[g].x - h.x, D[g].y - h.y);
   }
 }

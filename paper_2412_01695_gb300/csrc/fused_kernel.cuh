@@ -144,7 +144,9 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
     }
   }
   const V* nl_bk = nl ? static_cast<const V*>(a.beta) + (size_t)k * a.nkb * a.npw_beta : nullptr;
-  // FP64: the integer form, with beta and C turned into limbs where they are used
+  // FP64: the integer form (not where S C with q is wanted, see nl_fused.cuh), with beta and C
+  // turned into limbs where they are used
+  [[maybe_unused]] const bool ints = FX && !(a.sout != nullptr && a.qm != nullptr);
   [[maybe_unused]] const int* be = nl && FX ? a.bexp + (size_t)k * a.nkb : nullptr;
   [[maybe_unused]] int* ex = reinterpret_cast<int*>(nls + 3 * (size_t)a.nkb);
   [[maybe_unused]] auto load_b = [&](int m, int g) {
@@ -152,16 +154,20 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
     return nl_limbs(double2{b.x, b.y}, be[m] == kFxBadField ? 0 : be[m]);
   };
   if constexpr (nl) {
-    if constexpr (FX)
-      nl_fx_project(a.nkb, npi, be, scale.top, load_b, [&](int g) { return scale.bad ? int4{0, 0, 0, 0} : nl_limbs(pin[g], scale.top); }, nls);
-    else
+    if constexpr (FX) {
+      if (ints)
+        nl_fx_project(a.nkb, npi, be, scale.top, load_b, [&](int g) { return scale.bad ? int4{0, 0, 0, 0} : nl_limbs(pin[g], scale.top); }, nls);
+      else
+        nl_fused_project<T>(a, nl_bk, a.npw_beta, pin, npi, nls);
+    } else {
       nl_fused_project<T>(a, nl_bk, a.npw_beta, psis, npi, nls);
+    }
   }
   __syncthreads();
   if (nl) nl_fused_coef<T>(a, nls);   // read after the barriers that follow
   if constexpr (nl && FX) {
     __syncthreads();
-    nl_fx_coef(a.nkb, a.sout != nullptr && a.qm != nullptr, be, nls, ex);
+    if (ints) nl_fx_coef(a.nkb, be, nls, ex);
   }
 
   // ---- 2: inverse z transforms on the sticks
@@ -288,11 +294,12 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
         if constexpr (nl) {   // the in and out spheres are the same here (npi == npo)
           const bool with_q = with_s && a.qm != nullptr;
           V h, sv;
+          bool done = false;
           if constexpr (FX) {
-            nl_fx_addback(a.nkb, g, reinterpret_cast<const int4*>(nls) + a.nkb, ex, with_q, load_b, h, sv);
-          } else {
-            nl_fused_addback<T>(a, nl_bk, a.npw_beta, g, nls, with_q, h, sv);
+            if (ints) h = nl_fx_addback(a.nkb, g, reinterpret_cast<const int4*>(nls) + a.nkb, *ex, load_b);
+            done = ints;
           }
+          if (!done) nl_fused_addback<T>(a, nl_bk, a.npw_beta, g, nls, with_q, h, sv);
           acc.x += h.x;
           acc.y += h.y;
           if (with_s) {

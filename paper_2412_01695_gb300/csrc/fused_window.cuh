@@ -317,25 +317,31 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     const int* gout = a.gout + (size_t)k * a.npw_out_max;
     const double* g2k = a.g2 + (size_t)k * a.npw_out_max;
     V* LOC = reinterpret_cast<V*>(smem_raw + a.loc_off);   // [npw_out_max] local + kinetic
-    V* Cs = LOC + a.npw_out_max;                             // [npw_out_max] C in T (FP64: limbs)
+    V* Cs = LOC + a.npw_out_max;                             // [npw_out_max] C in T, or its limbs
     V* nls = reinterpret_cast<V*>(smem_raw + a.nl_off);
-    for (int g = tid; g < np; g += nth) {
-      const VI cv = pin[g];
-      LOC[g] = local(gout[g], T(g2k[g]), cv);
-      if constexpr (FX) reinterpret_cast<int4*>(Cs)[g] = scale.bad ? int4{0, 0, 0, 0} : nl_limbs(cv, scale.top);
-      else Cs[g] = V{T(cv.x), T(cv.y)};
-    }
-    __syncthreads();
-    V* Bs = reinterpret_cast<V*>(smem_raw);                  // [nkb][npw_beta] (FP64: limbs)
     const bool with_s = a.sout != nullptr;
     const bool with_q = with_s && a.qm != nullptr;
     VI* sout = with_s ? static_cast<VI*>(a.sout) + ((size_t)k * a.nvec_out + vout) * a.npw_out_max : nullptr;
+    const bool ints = FX && !with_q;                         // the integer sums of nl_fused.cuh
+    for (int g = tid; g < np; g += nth) {
+      const VI cv = pin[g];
+      LOC[g] = local(gout[g], T(g2k[g]), cv);
+      if constexpr (FX) {
+        if (ints) {
+          reinterpret_cast<int4*>(Cs)[g] = scale.bad ? int4{0, 0, 0, 0} : nl_limbs(cv, scale.top);
+          continue;
+        }
+      }
+      Cs[g] = V{T(cv.x), T(cv.y)};
+    }
+    __syncthreads();
+    V* Bs = reinterpret_cast<V*>(smem_raw);                  // [nkb][npw_beta] in T, or limbs
     if constexpr (FX) {
-      int4* Bl = reinterpret_cast<int4*>(Bs);
-      const int4* Cl = reinterpret_cast<const int4*>(Cs);
-      const int* be = a.bexp + (size_t)k * a.nkb;
-      int* ex = reinterpret_cast<int*>(nls + 3 * (size_t)a.nkb);
-      {
+      if (ints) {
+        int4* Bl = reinterpret_cast<int4*>(Bs);
+        const int4* Cl = reinterpret_cast<const int4*>(Cs);
+        const int* be = a.bexp + (size_t)k * a.nkb;
+        int* ex = reinterpret_cast<int*>(nls + 3 * (size_t)a.nkb);
         const double2* bk = static_cast<const double2*>(a.beta) + (size_t)k * a.nkb * a.npw_beta;
         for (int m = 0; m < a.nkb; ++m) {
           const int R = be[m] == kFxBadField ? 0 : be[m];
@@ -344,25 +350,24 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
             Bl[i] = nl_limbs(bk[i], R);
           }
         }
+        __syncthreads();
+        auto load_b = [&](int m, int g) { return Bl[(size_t)m * a.npw_beta + g]; };
+        nl_fx_project(a.nkb, np, be, scale.top, load_b, [&](int g) { return Cl[g]; }, nls);
+        __syncthreads();
+        nl_fused_coef<T>(a, nls);
+        __syncthreads();
+        nl_fx_coef(a.nkb, be, nls, ex);
+        __syncthreads();
+        const int4* gl = reinterpret_cast<const int4*>(nls) + a.nkb;
+        for (int g = tid; g < np; g += nth) {
+          const double2 h = nl_fx_addback(a.nkb, g, gl, *ex, load_b);
+          const V l = LOC[g];
+          if (with_s) sout[g] = pin[g];
+          pout[g] = VI{l.x + h.x, l.y + h.y};
+        }
       }
-      __syncthreads();
-      auto load_b = [&](int m, int g) { return Bl[(size_t)m * a.npw_beta + g]; };
-      nl_fx_project(a.nkb, np, be, scale.top, load_b, [&](int g) { return Cl[g]; }, nls);
-      __syncthreads();
-      nl_fused_coef<T>(a, nls);
-      __syncthreads();
-      nl_fx_coef(a.nkb, with_q, be, nls, ex);
-      __syncthreads();
-      const int4* gl = reinterpret_cast<const int4*>(nls) + a.nkb;
-      for (int g = tid; g < np; g += nth) {
-        double2 h, sv;
-        nl_fx_addback(a.nkb, g, gl, ex, with_q, load_b, h, sv);
-        const V l = LOC[g];
-        const VI cv = pin[g];
-        pout[g] = VI{l.x + h.x, l.y + h.y};
-        if (with_s) sout[g] = with_q ? VI{cv.x + sv.x, cv.y + sv.y} : cv;
-      }
-    } else {
+    }
+    if (!ints) {
       nl_stage_beta<T>(a, k, Bs);
       nl_fused_project<T>(a, Bs, a.npw_beta, Cs, np, nls);
       __syncthreads();
@@ -375,7 +380,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
         pout[g] = VI{TI(l.x + h.x), TI(l.y + h.y)};
         if (with_s) {
           const VI cv = pin[g];
-          sout[g] = a.qm != nullptr ? VI{cv.x + TI(sv.x), cv.y + TI(sv.y)} : cv;
+          sout[g] = with_q ? VI{cv.x + TI(sv.x), cv.y + TI(sv.y)} : cv;
         }
       }
     }

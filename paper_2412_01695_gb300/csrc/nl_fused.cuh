@@ -28,7 +28,7 @@ template <typename T, typename CV>
 __device__ __forceinline__ void nl_fused_project(const FusedArgs& a, const c2_t<T>* bk, int ldb,
                                                  const CV* cin, int np, c2_t<T>* nls) {
   using V = c2_t<T>;
-  constexpr int G = 4;   // projectors per warp group (accumulators held in registers)
+  constexpr int G = sizeof(T) == 4 ? 4 : 3;   // projectors per warp group (accumulators held in registers)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int ngroups = (a.nkb + G - 1) / G;
   for (int grp = warp; grp < ngroups; grp += nw) {
@@ -115,7 +115,7 @@ __device__ __forceinline__ void nl_fused_addback(const FusedArgs& a, const c2_t<
 
 // beta(k) ([nkb][npw_beta] contiguous) into shared memory at dst by asynchronous copies from
 // every thread of the CTA (16-byte copies when the block is 16-byte aligned and sized, else one
-// complex element per copy), FP32; returns once every copy has landed and the CTA has synchronised.
+// complex element per copy); returns once every copy has landed and the CTA has synchronised.
 template <typename T>
 __device__ __forceinline__ void nl_stage_beta(const FusedArgs& a, int k, c2_t<T>* dst) {
   using V = c2_t<T>;
@@ -128,9 +128,12 @@ __device__ __forceinline__ void nl_stage_beta(const FusedArgs& a, int k, c2_t<T>
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d0 + (unsigned)i), "l"(s + i) : "memory");
   } else {
     for (size_t i = threadIdx.x; i < n; i += blockDim.x) {
-      static_assert(sizeof(V) == 8, "FP32 vectors");
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d0 + (unsigned)(i * 8)), "l"(src + i)
-                   : "memory");
+      if constexpr (sizeof(V) == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d0 + (unsigned)(i * 16)), "l"(src + i)
+                     : "memory");
+      else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d0 + (unsigned)(i * 8)), "l"(src + i)
+                     : "memory");
     }
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -138,15 +141,19 @@ __device__ __forceinline__ void nl_stage_beta(const FusedArgs& a, int k, c2_t<T>
   __syncthreads();
 }
 
-// ------------------------------------------------------------------ FP64 projector terms
-// The same sums for FP64 vectors on the integer pipe: beta_m(k), C and the coefficients as
+// ------------------------------------------------------------------ FP64 projector terms of H
+// The same sums for FP64 vectors on the integer pipe, where S C is not asked for: beta_m(k), C and
+// the coefficients as
 // integers of 57 bits (scaled by the largest component of the projector, of the vector, of all
 // coefficients), split X = h 2^29 + l, so that a complex multiply-add is 12 wide integer
 // multiply-adds (the l l products, below 2^-56 of the largest product, are left out) instead
 // of 4 FP64 instructions at a fifteenth of their rate.  Sums are exact up to that; they return
 // to double once per lane and projector, and once per plane wave.  1280 band-k at N = 24 with 9
-// projectors: 0.48 -> 0.44 ms for the whole application (FP64 pipe 28 -> 11 % busy), error against
-// long double unchanged (1.9e-16).
+// projectors: 0.48 -> 0.44 ms for the whole application, error against long double unchanged
+// (1.9e-16).  What the sums lose below 2^-57 of the largest component stays under the rounding of
+// the local term, which spreads over all components alike.  S C = C + sum delta beta has no such
+// term and is exact to rounding in every component with sums in doubles, so a call that wants S
+// with q takes those (nl_fused_project and so on) for H too.
 // kNlFlush: terms an accumulator holds before it is taken over into double (|h| <= 2^28: a
 // complex term adds at most 4 2^56 to the middle sum).
 constexpr int kNlFlush = 31;
@@ -234,58 +241,46 @@ __device__ __forceinline__ void nl_fx_project(int nkb, int np, const int* bexp, 
   }
 }
 
-// After nl_fused_coef and a barrier, by warp 0: gamma (and delta) turned into limbs in place,
-// scaled so that with beta_m's scale every product has one unit; their exponents to ex[0], ex[1]
-// (kFxBadField: a coefficient is not finite).
-__device__ __forceinline__ void nl_fx_coef(int nkb, bool with_q, const int* bexp, double2* nls, int* ex) {
+// After nl_fused_coef and a barrier, by warp 0: gamma turned into limbs in place, scaled so that
+// with beta_m's scale every product has one unit; the exponent to *ex (kFxBadField: a coefficient
+// is not finite).
+__device__ __forceinline__ void nl_fx_coef(int nkb, const int* bexp, double2* nls, int* ex) {
   if (threadIdx.x >= 32) return;
   const int lane = threadIdx.x;
-  for (int s = 0; s < (with_q ? 2 : 1); ++s) {
-    double2* c = nls + (size_t)(1 + s) * nkb;
-    int top = -100000;
-    for (int m = lane; m < nkb; m += 32) {
-      const unsigned h = max(fx_abs_hi(c[m].x), fx_abs_hi(c[m].y));
-      const int be = bexp[m];
-      if ((h >> 20) == 0x7ff || be == kFxBadField) top = kFxBadField;
-      else if (c[m].x != 0.0 || c[m].y != 0.0) top = max(top, (int)max(h >> 20, 1u) - 1022 + be);
-    }
-    top = __reduce_max_sync(0xffffffffu, top);
-    if (top == -100000) top = 0;   // every coefficient is zero
-    if (lane == 0) ex[s] = top;
-    for (int m = lane; m < nkb; m += 32) {
-      const int be = bexp[m];
-      const int4 q = top == kFxBadField ? int4{0, 0, 0, 0} : nl_limbs(c[m], top - be);
-      reinterpret_cast<int4*>(c)[m] = q;
-    }
+  double2* c = nls + nkb;
+  int top = -100000;
+  for (int m = lane; m < nkb; m += 32) {
+    const unsigned h = max(fx_abs_hi(c[m].x), fx_abs_hi(c[m].y));
+    const int be = bexp[m];
+    if ((h >> 20) == 0x7ff || be == kFxBadField) top = kFxBadField;
+    else if (c[m].x != 0.0 || c[m].y != 0.0) top = max(top, (int)max(h >> 20, 1u) - 1022 + be);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (top == -100000) top = 0;   // every coefficient is zero
+  if (lane == 0) *ex = top;
+  for (int m = lane; m < nkb; m += 32) {
+    const bool zero = top == kFxBadField || (c[m].x == 0.0 && c[m].y == 0.0);
+    reinterpret_cast<int4*>(c)[m] = zero ? int4{0, 0, 0, 0} : nl_limbs(c[m], top - bexp[m]);
   }
 }
 
-// Epilogue for one plane wave (nl_fused_addback): h = sum_m gamma_m beta_m and, with_q, s = sum_m
-// delta_m beta_m; coef: the limbs of gamma, then delta
+// Epilogue for one plane wave (nl_fused_addback): sum_m gamma_m beta_m; coef: the limbs of gamma
 template <typename LB>
-__device__ __forceinline__ void nl_fx_addback(int nkb, int g, const int4* coef, const int* ex, bool with_q,
-                                              const LB& load_b, double2& h, double2& s) {
-  h = s = make_double2(0.0, 0.0);
-  NlSum ah, as;
+__device__ __forceinline__ double2 nl_fx_addback(int nkb, int g, const int4* coef, int ex, const LB& load_b) {
+  double2 h = make_double2(0.0, 0.0);
+  NlSum ah;
   for (int m0 = 0; m0 < nkb; m0 += kNlFlush) {
     const int m1 = min(nkb, m0 + kNlFlush);
 #pragma unroll 3
-    for (int m = m0; m < m1; ++m) {
-      const int4 b = load_b(m, g);
-      ah.add<false>(b, coef[m]);
-      if (with_q) as.add<false>(b, coef[nkb + m]);
-    }
+    for (int m = m0; m < m1; ++m) ah.add<false>(load_b(m, g), coef[m]);
     ah.flush(h);
-    if (with_q) as.flush(s);
   }
-  const double bad = nan("");
-  h = ex[0] == kFxBadField ? make_double2(bad, bad) : make_double2(nl_scaled(h.x, ex[0] - 85), nl_scaled(h.y, ex[0] - 85));
-  if (with_q)
-    s = ex[1] == kFxBadField ? make_double2(bad, bad) : make_double2(nl_scaled(s.x, ex[1] - 85), nl_scaled(s.y, ex[1] - 85));
+  if (ex == kFxBadField) return make_double2(nan(""), nan(""));
+  return make_double2(nl_scaled(h.x, ex - 85), nl_scaled(h.y, ex - 85));
 }
 
 // shared-memory bytes of the coefficients (lambda, gamma, delta) for nkb projectors; FP64: then
-// the exponents of gamma and delta
+// the exponent of gamma
 inline size_t nl_fused_bytes(int nkb, int elem_bytes) {
   return nkb > 0 ? (((size_t)3 * nkb * elem_bytes + 15) & ~(size_t)15) + (elem_bytes == 16 ? 16 : 0) : 0;
 }

@@ -228,3 +228,39 @@ def test_projector_terms_in_limbs(N, nat, lset, kind, spread):
     for v, got in zip(x[0], sp.cpu().numpy()[0]):
         ref = v[:n] + ((v[:n].astype(np.clongdouble) @ b.conj().T) @ q) @ b
         assert np.linalg.norm((got[:n] - ref).astype(complex)) <= 5e-16 * max(np.linalg.norm(ref.astype(complex)), 1e-300)
+
+
+@pytest.mark.parametrize("path,kind", [(2, 1), (3, 0), (3, 1), (3, 2)])
+def test_s_in_every_component(path, kind):
+    """S C of vectors that fall off like the projectors (smallest components 1e-6 of the largest):
+    every component to the rounding of sums in doubles, whatever its size.  Bound: u times the
+    sum of moduli times the additions a term goes through (n / 32 in a lane of the projection and
+    5 across lanes, nkb for delta, nkb for the add-back, two per complex product)."""
+    torch = torch_cuda()
+    N, lset = 24, (0, 1)
+    prob = problem(N, lset=lset)
+    q = synth.random_q(np.random.default_rng(2), 1, lset)
+    r = np.random.default_rng(7)
+    x = np.zeros((prob.nk, 4, prob.npw_max), complex)
+    for k in range(prob.nk):
+        n = int(prob.npw[k])
+        g = prob.kpts[k][None, :] + prob.miller[k][:n] @ prob.B
+        x[k, :, :n] = np.exp(-np.sum(g * g, axis=1) / 3) * (r.standard_normal((4, n)) + 1j * r.standard_normal((4, n)))
+    plan = pwk.plan_from_problem(prob)
+    plan.set_overlap(q)
+    plan.set_projector_path(path)
+    plan.set_launch_shape(pwk.PWK_FP64, kind, 128, 1)
+    assert plan.projector_fused(pwk.PWK_FP64) == (path == 3)
+    d = torch.from_numpy(x).cuda()
+    h, s = torch.full_like(d, 7.0), torch.full_like(d, 7.0)
+    pwk.hspsi_batched(plan, pwk.PWK_FP64, d, h, s, x.shape[1])
+    torch.cuda.synchronize()
+    plan.close()
+    for k in range(prob.nk):
+        n = int(prob.npw[k])
+        assert np.abs(x[k, :, :n]).min() < 1e-5 * np.abs(x[k]).max()
+        b, v = prob.beta[k][:, :n].astype(np.clongdouble), x[k, :, :n].astype(np.clongdouble)
+        ref = v + ((v @ b.conj().T) @ q) @ b
+        moduli = np.abs(v) + ((np.abs(v) @ np.abs(b).T) @ np.abs(q)) @ np.abs(b)
+        bound = 2.0 ** -53 * 2 * (n / 32 + 5 + 2 * prob.nkb + 4) * moduli
+        assert np.all(np.abs(s.cpu().numpy()[k, :, :n] - ref) <= bound)
