@@ -484,10 +484,12 @@ static void use_kind(const pwk_plan* p, FusedArgs& a, int kind) {
 
 // Pick the launch shape (kernel kind, threads per CTA, l3 chunk L) of one precision, and
 // whether the projector terms run inside the local kernel or in separate kernels, by timing
-// them on a sample of the plan's k-points (8 zero vectors per k, up to 512 k-points in FP32
-// and 96 in FP64; the work of the kernels does not depend on the values).  Every shape of a
+// them on a sample of the plan's k-points (8 vectors per k of one finite value throughout, up to
+// 512 k-points in FP32 and 96 in FP64; the scale of a zero vector would take the FP64 kernels
+// another pass, no other value changes their work).  Every shape of a
 // kind gives bitwise the same result: the arithmetic of each line and the order of every
 // reduction do not depend on the shape.
+constexpr int kTuneByte = 0x3f;   // 0.747 in FP32, 4.8e-4 in FP64
 int autotune_shape(pwk_plan* p, int precision) {
   const int N = p->N;
   const int elem = precision == PWK_FP64 ? 16 : 8;
@@ -518,7 +520,7 @@ int autotune_shape(pwk_plan* p, int precision) {
     cudaGetLastError();
     return PWK_OK;   // no room to tune: keep the default
   }
-  cudaMemset(in, 0, bytes);
+  cudaMemset(in, kTuneByte, bytes);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -580,7 +582,7 @@ int autotune_shape(pwk_plan* p, int precision) {
     void* coef = nullptr;
     if (cudaMalloc(&in, bytes2) == cudaSuccess && cudaMalloc(&out, bytes2) == cudaSuccess &&
         cudaMalloc(&coef, (size_t)nk2 * nv2 * 2 * p->nkb * elem) == cudaSuccess) {
-      cudaMemset(in, 0, bytes2);
+      cudaMemset(in, kTuneByte, bytes2);
       FusedArgs b = hpsi_args(p, precision, in, out);
       b.nvec_in = b.nvec_out = nv2;
       NlArgs n = nl_args(p, precision, in, out, nullptr, nullptr, nullptr, nk2 * nv2, nv2, nv2, 0);
