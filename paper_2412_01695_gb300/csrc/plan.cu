@@ -882,19 +882,8 @@ int pwk_plan_set_launch_shape(pwk_plan* p, int precision, int kind, int threads,
   c.kind = kind;
   c.threads = threads;
   c.L = l3_chunk;
-  auto bytes = [&] {
-    return c.kind >= 1 ? window_smem_bytes(p->N, elem, c.L, p->self.nstick_max, c.kind == 2 ? threads / 32 : 1)
-                       : fused_smem_bytes(p->N, elem, p->self.nstick_max, p->self.P, c.L, p->npw_max);
-  };
-  c.smem = bytes();
-  // an FP64 window shape within a few KB of the limit (its line shifts) takes the next smaller
-  // chunk, or the CTA-wide kind: the same bits
-  const size_t slack = 2048;
-  if (precision == PWK_FP64 && kind >= 1 && c.smem > 227 * 1024 && c.smem <= 227 * 1024 + slack) {
-    if (c.L > 1) --c.L;
-    else c.kind = 1;
-    c.smem = bytes();
-  }
+  c.smem = kind >= 1 ? window_smem_bytes(p->N, elem, l3_chunk, p->self.nstick_max, kind == 2 ? threads / 32 : 1)
+                     : fused_smem_bytes(p->N, elem, p->self.nstick_max, p->self.P, l3_chunk, p->npw_max);
   if (c.smem > 227 * 1024) {
     set_error("shape needs more than 227 KB of shared memory");
     return PWK_ERR_UNSUPPORTED;

@@ -200,6 +200,36 @@ def test_every_launch_shape_gives_identical_results(precision):
     plan.close()
 
 
+@pytest.mark.parametrize("N", [18, 24, 27, 36])
+def test_launch_shape_is_the_one_asked_for(N):
+    """Every shape is either installed as asked or refused (-2) with the plan's shape unchanged,
+    also those a little above the shared-memory limit (N = 27 with 21 planes in FP64)."""
+    torch_cuda()
+    from paper_2412_01695_gb300 import pwk
+    A = synth.sc_lattice(7.5)
+    ecut = ((N // 4 + 0.4) * 2 * np.pi / 7.5) ** 2 * 0.9
+    k = synth.mp_grid(synth.reciprocal_rows(A), (1, 1, 1)) + 0.05
+    prob = synth.build_problem(A, np.zeros((1, 3)), (0,), N, ecut, k, 1, 1, with_psi=False)
+    plan = pwk.plan_from_problem(prob)
+    for precision in pwk.PRECISIONS.values():
+        refused = 0
+        for kind in (0, 1, 2):
+            for T in (96, 128, 192, 256):
+                for L in range(1, N + 1) if kind < 2 else (1, 2):
+                    before = plan.launch_shape(precision)
+                    try:
+                        plan.set_launch_shape(precision, kind, T, L)
+                    except pwk.PwkError as e:
+                        assert e.code == -2
+                        assert plan.launch_shape(precision) == before
+                        refused += 1
+                        continue
+                    shape = plan.launch_shape(precision)
+                    assert tuple(shape[:3]) == (kind, T, L) and shape[3] <= 227 * 1024
+        assert refused > 0 or N < 27 or precision != pwk.PWK_FP64
+    plan.close()
+
+
 @pytest.mark.parametrize("precision", ["fp32", "fp32_c128"])
 @pytest.mark.parametrize("cfg,nks,nb", [(2, 6, 20), (1, 8, 8), (4, 5, 12), (2, 3, 44), (3, 2, 40), (3, 2, 7),
                                        (3, 3, 64)])
