@@ -284,10 +284,11 @@ __global__ void __launch_bounds__(512, 2) rr_kernel(int nk, int ld, int nb, cons
   // (||C||_F from the lower triangle)
   {
     double f = 0.0;
-    for_lower(n, tid, nth, [&](int r, int c) {
-      const double2 v = C[r * ld + c];
-      f += (r == c ? 1.0 : 2.0) * (v.x * v.x + v.y * v.y);
-    });
+    if (tid < 256)   // the order of the sum does not depend on nth
+      for_lower(n, tid, 256, [&](int r, int c) {
+        const double2 v = C[r * ld + c];
+        f += (r == c ? 1.0 : 2.0) * (v.x * v.x + v.y * v.y);
+      });
     f = block_sum(f, red);
     const double big = 4.0 * sqrt(f) + 1.0;
     for_lower(n, tid, nth, [&](int r, int c) {
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(512, 2) rr_kernel(int nk, int ld, int nb, cons
   // ---- 3. Householder tridiagonalisation of the Hermitian C held in its lower triangle;
   //      v_j stored in C[j+1..n-1][j] with v[0] = 1.  Per step: the product w = tau C22 v (P lanes
   //      per row, the upper half read through the lower triangle), the correction
-  //      w += alpha2 v (warp 0), and the rank-2 update of the lower triangle of C22, in which
+  //      w += alpha2 v (a warp per 32 rows), and the rank-2 update of the lower triangle of C22, in which
   //      warp 0 takes the first column and goes on to the next reflector (into the other buffer
   //      of vv) while the other warps do the rest.
   auto reflector = [&](int j, int buf) {   // warp 0; vv[buf][0..m) holds the updated column j below its diagonal
@@ -357,8 +358,8 @@ __global__ void __launch_bounds__(512, 2) rr_kernel(int nk, int ld, int nb, cons
     double2* C22 = C + (size_t)(j + 1) * ld + (j + 1);
     if (!skip) {
       // w = tau C22 v  (C22 = C[j+1.., j+1..], Hermitian, lower triangle stored)
-      int lp = 0;   // log2 of the lanes per row
-      while ((m << (lp + 1)) <= nth && lp < 4) ++lp;
+      int lp = 0;   // log2 of the lanes per row, as many as fill 256 threads
+      while ((m << (lp + 1)) <= 256 && lp < 4) ++lp;
       const int P = 1 << lp, p = tid & (P - 1);
       for (int rb = 0; rb < m; rb += nth >> lp) {   // uniform trip count: shuffles see every lane
         const int r = rb + (tid >> lp);
@@ -670,7 +671,9 @@ __global__ void __launch_bounds__(512, 2) rr_kernel(int nk, int ld, int nb, cons
     return;
   }
   // ---- 5. back-transform x = L^-H Q z of the selected vectors.  G lanes of one warp per
-  //      vector (G = 8 for nb <= 32, fewer for more vectors); lane c of a group holds the rows
+  //      vector, by nb and n (16 for nb <= 16 and n > 40, 8 for nb <= 32, fewer for more vectors;
+  //      one step more for n > 128: 40 vectors of n = 160, 128 problems, 16.4 -> 15.8 ms, 30 of n =
+  //      120 the other way where the batch is full); lane c of a group holds the rows
   //      r = c, c + G, c + 2G, ... of its vector, so a reflector on rows h+1..n-1 costs each
   //      lane about (n-h-1)/G row updates and a G-lane reduction, the triangular solve
   //      (column by column: x_r, then its share subtracted from the rows above) a broadcast
@@ -678,7 +681,8 @@ __global__ void __launch_bounds__(512, 2) rr_kernel(int nk, int ld, int nb, cons
   for (int j = tid; j < nb; j += nth) eps[k * nb + j] = lam[j];
   double2* E = ev + (size_t)k * ld * nb;
   {
-    const int G = nb <= nth / 16 && n > 40 ? 16 : nb <= nth / 8 ? 8 : nb <= nth / 4 ? 4 : nb <= nth / 2 ? 2 : 1;
+    const int fill = n > 128 ? 512 : 256;
+    const int G = nb <= fill / 16 && n > 40 ? 16 : nb <= fill / 8 ? 8 : nb <= fill / 4 ? 4 : nb <= fill / 2 ? 2 : 1;
     const int c = tid % G, lane = tid & 31, ngroups = nth / G;
     const int gbase = lane & ~(G - 1);   // lane of c = 0 in this group (G divides 32)
     auto first_row = [&](int lo) { return lo <= c ? c : c + G * ((lo - c + G - 1) / G); };
@@ -742,6 +746,10 @@ __global__ void __launch_bounds__(512, 2) rr_kernel(int nk, int ld, int nb, cons
   if (tid == 0 && status != nullptr) status[k] = PWK_OK;
 }
 
+// The bits of a problem depend on neither the number of problems nor the threads it gets: lanes per
+// row and per vector follow from n and nb (with lanes filled up to 512 threads instead of 256: 512
+// problems of n = 80 9.4 ms, against 8.7; 128 problems the same), the Frobenius norm is summed by
+// 256 threads, and every other sum by one thread or one warp.
 // Threads per problem: 512 where a CTA has an SM to itself and enough rows to fill them, 256 for
 // small problems and where several CTAs share an SM (n = 80, 20 vectors, 512 problems: 7.5 ms
 // with 256, 8.6 with 512; 128 problems: 2.64 with 512).  The Davidson passes the number of k-points

@@ -45,3 +45,30 @@ def test_block_edges(n, nprob):
         X = vec[p]
         np.testing.assert_allclose(X.conj().T @ S[p] @ X, np.eye(nev), atol=1e-9)
         assert np.max(np.linalg.norm(H[p] @ X - S[p] @ X * eig[p][None, :], axis=0)) < 1e-9 * scale * np.linalg.norm(S[p], 2) ** 0.5
+
+
+@pytest.mark.parametrize("n,nev", [(3, 2), (33, 8), (41, 5), (80, 20), (80, 40), (128, 32), (159, 40)])
+def test_bits_do_not_depend_on_the_batch(n, nev):
+    """A pencil alone, in a batch of 2 and in one of 305 (another number of threads per problem)
+    gives the same bits, with and without a dependent basis vector."""
+    torch = torch_cuda()
+    from paper_2412_01695_gb300 import pwk
+    rng = np.random.default_rng(n)
+    B = rng.standard_normal((2, n, 2 * n)) + 1j * rng.standard_normal((2, n, 2 * n))
+    if n > 4:
+        B[1, n - 2] = 0.5 * B[1, 0] - 2j * B[1, 1]
+    A = rng.standard_normal((2 * n, 2 * n)) + 1j * rng.standard_normal((2 * n, 2 * n))
+    H, S = B.conj() @ (A + A.conj().T) @ np.swapaxes(B, 1, 2), B.conj() @ np.swapaxes(B, 1, 2)
+    Hd, Sd = torch.from_numpy(H).cuda(), torch.from_numpy(S).cuda()
+    ref = None
+    for nprob in (2, 305):
+        reps = (nprob + 1) // 2
+        eig, vec = pwk.eigh_batched(Hd.repeat(reps, 1, 1)[:nprob].contiguous(),
+                                    Sd.repeat(reps, 1, 1)[:nprob].contiguous(), nev)
+        if ref is None:
+            ref = eig, vec
+        for p in range(2):
+            assert bool((eig[p::2] == ref[0][p]).all()) and bool((vec[p::2] == ref[1][p]).all()), (nprob, p)
+    for p in range(2):
+        eig, vec = pwk.eigh_batched(Hd[p:p + 1].contiguous(), Sd[p:p + 1].contiguous(), nev)
+        assert torch.equal(eig[0], ref[0][p]) and torch.equal(vec[0], ref[1][p])
