@@ -34,6 +34,7 @@
 // orthonormal to 1e-8, mark it PWK_ERR_NUMERIC.
 #include <cmath>
 
+#include "recip.cuh"
 #include "solvers.h"
 
 namespace pwk {
@@ -70,22 +71,6 @@ __device__ __forceinline__ void cfms_c(double2& s, double2 a, double2 b) {   // 
   s.x = fma(-a.y, b.y, s.x);
   s.y = fma(-a.y, b.x, s.y);
   s.y = fma(a.x, b.y, s.y);
-}
-
-// 1 / x and 1 / sqrt(x) to about an ulp: the hardware approximation (20 bits) and two Newton
-// steps.  x is normal and not near the ends of the range (pivots are clamped away from zero).
-__device__ __forceinline__ double fast_rcp(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(fma(-x, r, 1.0), r, r);
-  return fma(fma(-x, r, 1.0), r, r);
-}
-__device__ __forceinline__ double fast_rsqrt(double x) {
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double h = 0.5 * x;
-  r = fma(fma(-h * r, r, 0.5), r, r);
-  return fma(fma(-h * r, r, 0.5), r, r);
 }
 
 // Visit every (r, c) with 0 <= c <= r < m once, spread over the block: rows p and m-1-p are
