@@ -102,9 +102,6 @@ PWK_FX_HD int2 fx_pair(long long v) {
   return int2{l.hp, l.ls};
 }
 
-// v / 2^d rounded to nearest (d = 0 .. 62)
-PWK_FX_HD long long fx_shr(long long v, int d) { return (v + ((1LL << d) >> 1)) >> d; }
-
 // Largest bit length a value may have before a forward transform of length n: the sums of n
 // terms of modulus sqrt(2) |component| stay below 2^kFxBits.
 __host__ __device__ constexpr int fx_cap(int n) {

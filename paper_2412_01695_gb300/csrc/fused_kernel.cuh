@@ -32,25 +32,18 @@
 
 namespace pwk {
 
-// Load the N contiguous values of one V(r) x-line (layout [l2][l3][l1], l1 fastest) with
-// 16-byte vector loads when the line is 16-byte aligned (N * sizeof(T) a multiple of 16).
-template <typename T, int N>
-__device__ __forceinline__ void load_vline(const T* __restrict__ p, T (&w)[N]) {
-  constexpr int VEC = 16 / sizeof(T);
-  if constexpr ((N * sizeof(T)) % 16 == 0) {
-    using VT = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-    const VT* q = reinterpret_cast<const VT*>(p);
-    PWK_SFOR(N / VEC, j, {
-      const VT v = __ldg(q + j);
-      if constexpr (sizeof(T) == 4) {
-        w[4 * j] = v.x;
-        w[4 * j + 1] = v.y;
-        w[4 * j + 2] = v.z;
-        w[4 * j + 3] = v.w;
-      } else {
-        w[2 * j] = v.x;
-        w[2 * j + 1] = v.y;
-      }
+// Load the N contiguous values of one FP32 V(r) x-line (layout [l2][l3][l1], l1 fastest) with
+// 16-byte vector loads when the line is 16-byte aligned (N a multiple of 4).
+template <int N>
+__device__ __forceinline__ void load_vline(const float* __restrict__ p, float (&w)[N]) {
+  if constexpr (N % 4 == 0) {
+    const float4* q = reinterpret_cast<const float4*>(p);
+    PWK_SFOR(N / 4, j, {
+      const float4 v = __ldg(q + j);
+      w[4 * j] = v.x;
+      w[4 * j + 1] = v.y;
+      w[4 * j + 2] = v.z;
+      w[4 * j + 3] = v.w;
     });
   } else {
     PWK_SFOR(N, j, w[j] = __ldg(p + j));
@@ -213,7 +206,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
         sx[l2 * L + c] = (unsigned char)fx_v_product<N>(x, static_cast<const int2*>(a.V) + vline, y);
       } else {
         A w[N];
-        load_vline<A, N>(static_cast<const A*>(a.V) + vline, w);
+        load_vline<N>(static_cast<const float*>(a.V) + vline, w);
         PWK_SFOR(N, l1, {
           const VA u = x[OutSlot<N, l1>::value];
           y[l1] = VA{u.x * w[l1], u.y * w[l1]};

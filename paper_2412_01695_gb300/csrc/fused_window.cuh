@@ -169,7 +169,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
         const int l2 = t / lc, c = t - l2 * lc;
         // V(r) of the line is requested first: its latency hides behind the inverse transform
         A w[N];
-        load_vline<A, N>(static_cast<const A*>(a.V) + ((size_t)l2 * N + l0 + c) * N, w);
+        load_vline<N>(static_cast<const float*>(a.V) + ((size_t)l2 * N + l0 + c) * N, w);
         VA x[N], y[N];
         VA* yl = Yc + (size_t)l2 * L + c;
         PWK_SFOR(N, i, x[i] = Wn::in(i) ? yl[(size_t)Wn::idx(i) * yps] : VA{A(0), A(0)});

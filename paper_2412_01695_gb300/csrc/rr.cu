@@ -42,10 +42,6 @@ namespace pwk {
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-__device__ __forceinline__ double2 cmulc(double2 a, double2 b) {  // conj(a) * b
-  return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
-__device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 // accumulate with two fused multiply-adds per real component (4 FP64 instructions per
 // complex multiply-add)
 __device__ __forceinline__ void cfma(double2& s, double2 a, double2 b) {   // s += a b
@@ -108,9 +104,6 @@ __device__ double block_sum(double v, double* red) {
   for (int i = 0; i < nw; ++i) s += red[i];
   __syncthreads();
   return s;
-}
-__device__ double2 block_sum2(double2 v, double* red) {
-  return make_double2(block_sum(v.x, red), block_sum(v.y, red));
 }
 
 // Rayleigh-Ritz of every active k (active[k] != 0).
