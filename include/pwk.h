@@ -47,7 +47,7 @@ extern "C" {
 #define PWK_ERR_NUMERIC (-7)     /* CG breakdown (d^T A d <= 0) or non-finite values */
 
 /* arithmetic of an H|psi> application */
-#define PWK_FP64 0        /* complex128 in/out, FP64 arithmetic                          */
+#define PWK_FP64 0        /* complex128 in/out, FP64 accuracy (see pwk_hpsi_batched)     */
 #define PWK_FP32 1        /* complex64 in/out, FP32 arithmetic                           */
 #define PWK_FP32_C128 2   /* complex128 in/out, FP32 arithmetic (mixed-precision inner)  */
 
@@ -101,10 +101,11 @@ int pwk_plan_set_launch_shape(pwk_plan* plan, int precision, int kind, int threa
 
 /* How the nonlocal projector terms (Eqs. lambdah, gamma, finalnl; with q also delta_eq,
  * finals) are applied:
- *   0 (default)  automatic: path 2, unless path 3 or (FP32 arithmetic) path 1 ran more than
- *                3 % faster when pwk_plan_create timed them for each precision as whole H
- *                applications of 32 bands on the plan's own k-points (then the faster of
- *                the two; pwk_plan_projector_choice tells);
+ *   0 (default)  automatic, from whole H applications of 32 bands on the plan's own k-points
+ *                that pwk_plan_create times for each precision.  FP32 arithmetic: path 2,
+ *                unless path 3 or 1 ran more than 3 % faster (then the faster of the two).
+ *                FP64: path 3, unless path 2 ran more than 3 % faster.
+ *                pwk_plan_projector_choice tells;
  *   1            separate kernels, both contractions of FP32 batched calls on whole k-points
  *                on the 5th-generation tensor cores where they apply (2 nkb <= 128, nb <= 128,
  *                tiles within shared memory; the S add-back stays on the CUDA cores): three
@@ -157,7 +158,15 @@ int pwk_supported_grid(int N);
  *   psi        device [nk][nb][npw_max] complex128 (complex64 for PWK_FP32)
  *   hpsi       device, same shape and type; may be the same pointer as psi (in place),
  *              must not otherwise overlap it
- * Three launches on `stream` (projections, local and kinetic terms, nonlocal add-back); the
+ * PWK_FP64: the 2-norm of the error of a band is that of FP64 transforms, about 2e-16 of the
+ * band's result (5e-16 at most in the tests).  The transforms, and with path 3 the projector sums
+ * of a call for H alone, run in 64-bit integers scaled by the vector, V(r) and the projectors as
+ * a whole: like a transform in FP64 they spread their rounding over all components alike, so a
+ * component far below the others is exact to the rounding of the largest, not of itself (S psi of
+ * pwk_hspsi_batched is exact to rounding in every component).  A vector with a component that is
+ * not finite gives NaN in all its components.
+ * One launch on `stream` with path 3, else three (projections, local and kinetic terms, nonlocal
+ * add-back); the
  * projector coefficients between them (2 nkb complex per band-k) take scratch for the call
  * from a stream-ordered memory pool the library keeps per device (memory returned to the
  * pool stays mapped for later calls).  Asynchronous on `stream`. */
@@ -315,6 +324,7 @@ int pwk_drho_batched(pwk_plan* plan_kq, pwk_plan* plan_k, int precision, const v
  *           S is dependent on the earlier ones) or PWK_ERR_NUMERIC (non-finite eigenvector)
  * A row j >= nev whose Cholesky pivot falls below 1e-6 S_jj is treated as dependent and left
  * out of the problem (its eigenvector entries are zero).  1 <= nev <= n <= 160.
+ * The results of a problem depend on its matrices, n and nev alone, bit for bit: not on nprob.
  * Allocates a workspace of 3 n^2 complex128 per problem for the call and synchronises
  * `stream` before returning. */
 int pwk_eigh_batched(int nprob, int n, int nev, const void* H, const void* S, double* eig,

@@ -61,8 +61,8 @@ __device__ __forceinline__ V drho_value(longlong2 q) { return V{__ll2double_rn(q
 
 // FP64 transforms run in the fixed point of fixed.cuh (inverse only, so each field keeps the one
 // scale of its vector); the values come back to double at the product.  768 pairs at N = 20: 1.05
-// ms with FP64 transforms, 0.43 with these; then bound by the product (ten FP64 instructions per
-// grid point, 57 % of that pipe) and the barriers between the passes.
+// ms with FP64 transforms, 0.42 with these; then bound by the conversions and the product (eight FP64
+// instructions per grid point, 53 % of that pipe) and the barriers between the passes.
 template <typename T, int N>
 __global__ void __launch_bounds__(256, drho_ctas<T, N>()) drho_kernel(DrhoArgs a) {
   using V = c2_t<T>;
@@ -241,7 +241,10 @@ __device__ __forceinline__ int warp_exponent(const double2* v, int np) {
 // P_c du = du - sum_v u_v <su_v|du> (su = S u, or u when S = 1), one CTA per (k, nu).  The two
 // contractions are the projector sums of nl_fused.cuh with the valence states as projectors, on
 // the integer pipe: with FP64 multiply-adds they held that pipe (85 % busy) for 113 us on 768 pairs
-// of 12 valence states.
+// of 12 valence states; now 83 us (21 %).  The components of P_c du carry 57 bits of the largest;
+// the transform that follows spreads its rounding over all of them alike.  drho against long double,
+// limbs (doubles), 3 and 12 valence states: flat vectors 3.3e-16 (3.4), 3.4 (3.8); falling off with
+// the kinetic energy 3.2 (3.3), 3.4 (3.8).
 __global__ void __launch_bounds__(256) conduction_kernel(int nocc, int np, const int* npw,
                                                          const double2* u, const double2* su,
                                                          const double2* du, double2* out) {

@@ -1,7 +1,7 @@
 // Fused local-potential kernel: one CTA applies the kinetic and local terms of H to one
 // band of one k-point with a single round trip to HBM (read C, write the local part of H C).
-// The nonlocal projector terms run as separate kernels around it (nonlocal.cu): their
-// projections over all bands of a k-point share one staged copy of beta(k).
+// The nonlocal projector terms run inside it (NL below) or as separate kernels around it
+// (nonlocal.cu), whose projections of several bands of a k-point share one staged copy of beta(k).
 //
 // Per work item (paper Sec. 2.2 and Sec. 4, Fig. 2 flow, here fused into one kernel):
 //   1. load C(G) and scatter it onto the z-sticks held in shared memory (Sec. 3 "sets the

@@ -615,9 +615,11 @@ int autotune_shape(pwk_plan* p, int precision) {
       }
       // near ties (timing noise) resolve the same way in every process: FP32 takes the separate
       // CUDA-core kernels unless another path is faster by more than 3 %.  FP64 takes the fused
-      // terms unless the separate kernels are: those hold the FP64 pipe, and on uneven lists with
-      // S they cost twice what this sample of whole band sets shows (H and S of 237 items at N =
-      // 27 with 8 projectors: 0.66 ms separate, 0.27 to 0.36 fused)
+      // terms unless the separate kernels are: whole sets of 32 bands are where those do best (they
+      // stage beta(k) once for eight bands).  Ten cells (N = 15 to 27, 1 to 16 projectors, 27 and
+      // 64 k-points), time of the separate over that of the fused form: 0.96 to 1.29 with 32 bands,
+      // 1.02 to 1.63 with 16, on uneven lists 1.14 to 2.7; with S as well 0.93 to 1.18, 0.99 to 1.60
+      // and 1.13 to 2.8.
       if (precision == PWK_FP64) {
         fused = tf <= 1.03f * ts;
       } else if (std::min(tf, tt) < 0.97f * ts) {

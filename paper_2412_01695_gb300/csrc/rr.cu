@@ -26,9 +26,10 @@
 // its serial parts as much: measured per phase at n = 80, 20 vectors, one CTA per SM (us, before ->
 // after the look-ahead, the blocked solves and 512 threads instead of 256): Cholesky 257 -> 208, X
 // 510 -> 307, C 514 -> 216, Householder 1516 -> 1026, eigenvalues 353 -> 265, inverse iteration
-// 200 -> 193, back-transform 411 -> 405; in all 3.80 -> 2.64 ms (FP64 pipe 45 -> 67 % busy).  n =
-// 32, 8 vectors: 0.83 -> 0.55 ms; n = 160, 40 vectors: 16.1 -> 13.4 ms; 512 problems of n = 80: 7.4
-// -> 7.5 ms.
+// 200 -> 193, back-transform 411 -> 405; in all 3.80 -> 2.64 ms (FP64 pipe 65 % busy).  n = 32, 8
+// vectors: 0.83 -> 0.55 ms; n = 160, 40 vectors: 16.1 -> 13.4 ms; 512 problems of n = 80: 7.4 -> 7.5
+// ms.  (Taken with lanes filled up to 512 threads; up to 256, as now: 2.66 ms for n = 80, 2 to 3 %
+// more at n = 160, 3 % less at n = 32.)
 // A dependent vector among the first nb (pivot below 1e-6 of its diagonal) marks the k-point
 // with status PWK_ERR_NOT_POSDEF; a non-finite eigenvector, or eigenvectors of T that are not
 // orthonormal to 1e-8, mark it PWK_ERR_NUMERIC.

@@ -196,11 +196,12 @@ SITES = 7.5 * np.array([[0, 0, 0], [0, 0.5, 0.5], [0.5, 0, 0.5], [0.5, 0.5, 0]])
 @pytest.mark.parametrize("kind", [0, 1])
 @pytest.mark.parametrize("spread", [0, 150])
 def test_projector_terms_in_limbs(N, nat, lset, kind, spread):
-    """The integer projector sums inside the FP64 kernel: one projector, more than the 31 an
-    accumulator holds in the add-back (36), more plane waves than it holds in a lane (1500 > 31 *
-    32), and projectors of very different size (2^-spread to 2^spread, the coefficients scaled
-    back).  H and S against long double; the bar is that of the H tests (the limbs hold 57 bits of
-    the largest component, the left-out products 2^-56 of the largest product)."""
+    """The projector sums inside the FP64 kernel, on the integer pipe (H alone) and in doubles (H
+    and S with q): one projector, more than the 31 an accumulator holds in the add-back (36), more
+    plane waves than it holds in a lane (1500 > 31 * 32), and projectors of very different size
+    (2^-spread to 2^spread, the coefficients scaled back).  H and S against long double; the bar is
+    that of the H tests (the limbs hold 57 bits of the largest component, the left-out products
+    2^-56 of the largest product)."""
     torch = torch_cuda()
     from paper_2412_01695_gb300 import pwk
     ecut = ((N // 4 + 0.4) * 2 * np.pi / 7.5) ** 2 * 0.9
@@ -220,9 +221,12 @@ def test_projector_terms_in_limbs(N, nat, lset, kind, spread):
     d = torch.from_numpy(x).cuda()
     h, sp = torch.full_like(d, complex(np.nan, np.nan)), torch.full_like(d, complex(np.nan, np.nan))
     pwk.hspsi_batched(plan, pwk.PWK_FP64, d, h, sp, x.shape[1])
+    alone = torch.full_like(d, complex(np.nan, np.nan))
+    pwk.hpsi_batched(plan, pwk.PWK_FP64, d, alone, x.shape[1])
     torch.cuda.synchronize()
     plan.close()
     check(prob, x, h.cpu().numpy())
+    check(prob, x, alone.cpu().numpy())
     n = int(prob.npw[0])
     b = prob.beta[0][:, :n].astype(np.clongdouble)
     for v, got in zip(x[0], sp.cpu().numpy()[0]):
