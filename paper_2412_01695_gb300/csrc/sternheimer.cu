@@ -970,11 +970,11 @@ extern "C" int pwk_sternheimer_cg_batched(pwk_plan* pq, pwk_plan* pk, int mode, 
   // mixed mode: the inner solves on FP32 vectors (fused step only)
   const size_t upd32_smem = (size_t)3 * np * sizeof(float2);
   const bool inner32 = fused_step && mode == PWK_FP32_C128;
-  if (inner32 && upd32_smem > 48 * 1024) {
+  if (inner32) {   // whatever the size: the kernels' static shared memory counts towards the 48 KB too
     cudaError_t e = allow_full_smem(cg_update32_kernel);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(cg_update32)");
   }
-  if (fused_step && upd_smem > 48 * 1024) {
+  if (fused_step) {
     cudaError_t e = allow_full_smem(cg_update_kernel);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(cg_update)");
   }

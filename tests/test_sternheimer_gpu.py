@@ -184,3 +184,26 @@ def test_single_occupied_band():
     pk, pq, psi_k, psi_q, eps_k, eps_q_all, Hq_all, alpha, dv = inp
     rc, x, iters, resid = run_gpu(pk, pq, psi_k, psi_q, eps_k, alpha, dv, "fp64")
     check(pk, pq, psi_k, psi_q, eps_k, eps_q_all, Hq_all, alpha, dv, x, resid, rc)
+
+
+@pytest.mark.parametrize("mode,ecut,npw", [("fp64", 21.5, (1248, 1536)), ("mixed", 25.9, (1685, 2048)),
+                                           ("fp64", 25.9, (1537, 2048)), ("mixed", 21.5, (1248, 1684))])
+def test_spheres_around_the_default_shared_memory_limit(mode, ecut, npw):
+    """The fused CG step keeps two FP64 (three FP32) vectors of npw in shared memory beside 9 KB of
+    its own: sphere sizes at which the vectors alone stay below the default limit of 48 KB and
+    all of it does not, and sizes on either side.  Every pair is positive definite (eps below the
+    spectrum)."""
+    A = synth.sc_lattice(9.4)
+    k = synth.mp_grid(synth.reciprocal_rows(A), (1, 1, 1)) + 0.03
+    p = synth.build_problem(A, np.zeros((1, 3)), (0,), 32, ecut, k, 2, 1, vamp=0.1)
+    n = int(p.npw[0])
+    assert npw[0] <= n <= npw[1]
+    eps = np.array([[-20.0, -20.1]])
+    dv = synth.dv_grid(synth.rng_for(1, "dv"), p.B, p.N, ecut)
+    rc, x, iters, resid = run_gpu(p, p, p.psi, p.psi, eps, np.ones(1), dv, mode)
+    assert rc == 0 and resid.max() <= TOL
+    H, dvt, P = ham.problem_h(p, 0, ham.grid_coefficients(p.V_r)), ham.grid_coefficients(dv), p.psi[0, :, :n]
+    dvpsi = st.dv_psi_dense(p.miller[0, :n], p.miller[0, :n], dvt, P)
+    for b in range(2):
+        rhs = st.rhs(dvpsi[b], P)
+        assert np.linalg.norm(st.operator(H, P, eps[0, b], 1.0) @ x[0, b, :n] - rhs) <= TOL * np.linalg.norm(rhs)
