@@ -78,15 +78,15 @@ PATH_NAMES = {1: "separate tensor-core kernels", 2: "separate CUDA-core kernels"
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of a kernel, from ncu captures
 # summarised under profiles/, with the digest of the sources they were captured at.
-# rr_kernel: a full-batch launch of the 64-k solve (11.04 MB) scaled by k-points to the
+# rr_kernel: a full-batch launch of the 64-k solve (10.61 MB) scaled by k-points to the
 # 512-k batch of the headline step.
 # The H|psi> kernels of the 512-k cell in FP32: mean of three launches.
 TRAFFIC = {
-    "rr_kernel": {"bytes": 8 * 11042560, "profile": "profiles/rr_kernel_davidson_fcc64k_20b.md",
-                  "sources": ["rr.cu", "solvers.h"], "digest": "88ebedd93321"},
+    "rr_kernel": {"bytes": 8 * (10562816 + 44288), "profile": "profiles/rr_kernel_davidson_fcc64k_20b.md",
+                  "sources": ["rr.cu", "solvers.h"], "digest": "561669374c49"},
     "fused_window_kernel<float,float,24,6>": {
-        "bytes": 48430848 + 4129195, "profile": "profiles/hpsi_step_kernels_fcc512k_20b_fp32.md",
-        "sources": ["fused_window.cuh", "fft_line.cuh", "hpsi_f32.cu"], "digest": "e8fae88693ee"},
+        "bytes": 48416683 + 4098645, "profile": "profiles/hpsi_step_kernels_fcc512k_20b_fp32.md",
+        "sources": ["fused_window.cuh", "fft_line.cuh", "hpsi_f32.cu"], "digest": "573ad38aa930"},
     "nl_project_kernel<float,float,9>": {
         "bytes": 65060011 + 12288, "profile": "profiles/hpsi_step_kernels_fcc512k_20b_fp32.md",
         "sources": ["nonlocal.cu"], "digest": "67c9475f7eb9"},
@@ -94,9 +94,9 @@ TRAFFIC = {
         "bytes": 66527147 + 159061, "profile": "profiles/hpsi_step_kernels_fcc512k_20b_fp32.md",
         "sources": ["nonlocal.cu"], "digest": "67c9475f7eb9"},
     "fused_window_kernel_nl<float,float,24,6>": {
-        "bytes": 68650069 + 11811669, "profile": "profiles/fused_window_kernel_nl_hpsi_fcc512k_20b_fp32.md",
+        "bytes": 68634965 + 11855189, "profile": "profiles/fused_window_kernel_nl_hpsi_fcc512k_20b_fp32.md",
         "sources": ["fused_window.cuh", "fft_line.cuh", "nl_fused.cuh", "hpsi_f32_nl.cu"],
-        "digest": "d9d6563f277a"},
+        "digest": "c7071c70bae3"},
 }
 
 
