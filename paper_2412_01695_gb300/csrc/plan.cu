@@ -190,13 +190,14 @@ __global__ void fx_field_kernel(int N, int ncomp, const double* in, const unsign
   }
 }
 
-// Exponents of the projectors, a warp each: every |component| < 2^exponent (kFxBadField: one is
-// not finite)
-__global__ void beta_exponent_kernel(int n, int npw_max, const double2* beta, int* bexp) {
+// Exponents of the projectors, a warp each: every |component| inside the sphere < 2^exponent
+// (kFxBadField: one is not finite)
+__global__ void beta_exponent_kernel(int n, int nkb, const int* npw, int npw_max, const double2* beta, int* bexp) {
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= n) return;   // uniform over the warp
   unsigned h = 0;
-  for (int g = lane; g < npw_max; g += 32) {
+  const int np = npw[i / nkb];
+  for (int g = lane; g < np; g += 32) {
     const double2 b = beta[(size_t)i * npw_max + g];
     h = max(h, max((unsigned)__double2hiint(b.x) & 0x7fffffffu, (unsigned)__double2hiint(b.y) & 0x7fffffffu));
   }
@@ -1022,7 +1023,7 @@ int pwk_plan_create(pwk_plan** out, const double* A, int N1, int N2, int N3, int
     to_f32_kernel<<<blocks_for(nb2), 256>>>(nb2, static_cast<const double*>(beta), (float*)p->d_beta32); note_launch();
     TRYC(cudaGetLastError(), "beta to f32");
     TRY(plan_alloc(p, (void**)&p->d_bexp, sizeof(int) * (size_t)nk * nkb));
-    beta_exponent_kernel<<<blocks_for((size_t)nk * nkb, 8), 256>>>(nk * nkb, npw_max, static_cast<const double2*>(beta), p->d_bexp); note_launch();
+    beta_exponent_kernel<<<blocks_for((size_t)nk * nkb, 8), 256>>>(nk * nkb, nkb, p->d_npw, npw_max, static_cast<const double2*>(beta), p->d_bexp); note_launch();
     TRYC(cudaGetLastError(), "beta_exponent_kernel");
     std::vector<float> D32(p->h_D.begin(), p->h_D.end());
     TRY(plan_alloc(p, (void**)&p->d_D, sizeof(double) * nkb * nkb));

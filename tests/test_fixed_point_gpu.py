@@ -166,6 +166,21 @@ def test_s_of_a_non_finite_vector(bad, path, kind):
         assert np.all(np.isfinite(out[[0, 1, 3]]))
 
 
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("padding", [np.nan, 2.0 ** 600])
+def test_padding_of_the_projectors_does_not_enter(kind, padding):
+    """What lies beyond a sphere in beta takes no part in the scale of a projector: the same bits
+    as with zeros there."""
+    k = synth.mp_grid(B, (2, 2, 2))[:2] * np.array([[1.0], [0.3]]) + 0.05
+    prob = synth.build_problem(A, np.zeros((1, 3)), (0, 1), 16, 20.0, k, 4, 1, with_psi=False)
+    short = int(np.argmin(prob.npw))
+    assert prob.npw[short] < prob.npw_max
+    x = vectors(prob)
+    ref = apply(prob, x, (kind, 128, 1), path=3)
+    prob.beta[short, :, prob.npw[short]:] = padding
+    assert np.array_equal(apply(prob, x, (kind, 128, 1), path=3), ref)
+
+
 @pytest.mark.parametrize("field", ["zero", "constant", "large", "tiny", "spike", "nan"])
 def test_fields(field):
     N = 20
