@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 && N <= 25 ? 384 : 256) fused_k
   const V* nl_bk = nl ? static_cast<const V*>(a.beta) + (size_t)k * a.nkb * a.npw_beta : nullptr;
   // FP64: the integer form (not where S C with q is wanted, see nl_fused.cuh), with beta and C
   // turned into limbs where they are used
-  [[maybe_unused]] const bool ints = FX && !(a.sout != nullptr && a.qm != nullptr);
+  [[maybe_unused]] const bool ints = FX && a.nl_ints && !(a.sout != nullptr && a.qm != nullptr);
   [[maybe_unused]] const int* be = nl && FX ? a.bexp + (size_t)k * a.nkb : nullptr;
   [[maybe_unused]] int* ex = reinterpret_cast<int*>(nls + 3 * (size_t)a.nkb);
   [[maybe_unused]] auto load_b = [&](int m, int g) {

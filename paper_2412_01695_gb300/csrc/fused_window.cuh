@@ -323,7 +323,7 @@ __device__ __forceinline__ void window_body(const FusedArgs& a, int k, int vin, 
     const bool with_s = a.sout != nullptr;
     const bool with_q = with_s && a.qm != nullptr;
     VI* sout = with_s ? static_cast<VI*>(a.sout) + ((size_t)k * a.nvec_out + vout) * a.npw_out_max : nullptr;
-    const bool ints = FX && !with_q;                         // the integer sums of nl_fused.cuh
+    const bool ints = FX && a.nl_ints && !with_q;            // the integer sums of nl_fused.cuh
     for (int g = tid; g < np; g += nth) {
       const VI cv = pin[g];
       LOC[g] = local(gout[g], T(g2k[g]), cv);

@@ -151,9 +151,10 @@ __device__ __forceinline__ void nl_stage_beta(const FusedArgs& a, int k, c2_t<T>
 // to double once per lane and projector, and once per plane wave.  1280 band-k at N = 24 with 9
 // projectors: 0.48 -> 0.44 ms for the whole application, error against long double unchanged
 // (1.9e-16).  What the sums lose below 2^-57 of the largest component stays under the rounding of
-// the local term, which spreads over all components alike.  S C = C + sum delta beta has no such
-// term and is exact to rounding in every component with sums in doubles, so a call that wants S
-// with q takes those (nl_fused_project and so on) for H too.
+// the local term, which spreads over all components alike; a plan whose V is weaker than its
+// projectors (choose_projector_sums in plan.cu) takes the sums in doubles.  S C = C + sum delta beta
+// has no such term and is exact to rounding in every component with sums in doubles, so a call
+// that wants S with q takes those (nl_fused_project and so on) for H too.
 // kNlFlush: terms an accumulator holds before it is taken over into double (|h| <= 2^28: a
 // complex term adds at most 4 2^56 to the middle sum).
 constexpr int kNlFlush = 31;

@@ -221,6 +221,33 @@ __global__ void sum_kernel(size_t n, const double* in, double* out) {
 
 static int blocks_for(size_t n, int t = 256) { return (int)((n + t - 1) / t); }
 
+// Whether H alone takes the integer projector sums in FP64: those are exact to 2^-57 of the largest
+// product gamma beta, so they need a local term whose rounding is at least that large in every
+// component, max |V| >= w = sum_mn |D_mn| max |beta_m| max |beta_n| (the maxima over all k, rounded
+// up to powers of two; the local matrix has elements up to max |V|, the projectors' up to w).
+// vhi: the high word of max |V|.  Vectors that fall off with the kinetic energy, N = 24, 9
+// projectors, largest error of a component over its size: max |V| = 31 w, 1.9e-14 (3e-14 with a
+// steeper vector); max |V| = w / 3, 3.4e-14; with FP64 transforms and sums 1.0e-13 to 1.7e-13 in
+// both.  V = 0: 6e-13 (6e-12), with sums in doubles 2.4e-15 (9.4e-15).
+static int choose_projector_sums(pwk_plan* p, unsigned vhi) {
+  if (p->nkb == 0) return PWK_OK;
+  std::vector<int> e((size_t)p->nk * p->nkb);
+  cudaError_t err = cudaMemcpy(e.data(), p->d_bexp, e.size() * sizeof(int), cudaMemcpyDeviceToHost);
+  if (err != cudaSuccess) return cuda_fail(err, "cudaMemcpy(bexp)");
+  for (size_t i = p->nkb; i < e.size(); ++i) e[i % p->nkb] = std::max(e[i % p->nkb], e[i]);
+  double w = 0.0;   // infinite where a projector is not finite: sums in doubles
+  for (int m = 0; m < p->nkb; ++m)
+    for (int n = 0; n < p->nkb; ++n) {
+      const double d = std::fabs(p->h_D[(size_t)m * p->nkb + n]);
+      if (d != 0.0) w += std::ldexp(std::ldexp(d, e[m]), e[n]);
+    }
+  const unsigned long long bits = (unsigned long long)vhi << 32;
+  double vmax;
+  std::memcpy(&vmax, &bits, sizeof(vmax));
+  p->nl_ints = vmax >= w;
+  return PWK_OK;
+}
+
 int launch_fx_field(int N, int ncomp, const double* field, void* pairs, unsigned* hmax, int* vexp, cudaStream_t st) {
   const size_t n3 = (size_t)N * N * N;
   cudaError_t e = cudaMemsetAsync(hmax, 0, sizeof(unsigned), st);
@@ -443,6 +470,7 @@ static void set_fused_nl(const pwk_plan* p, int precision, FusedArgs& a, void* s
   a.qm = f64 ? static_cast<const void*>(p->d_q) : static_cast<const void*>(p->d_q32);
   a.sout = sout;
   a.bexp = p->d_bexp;
+  a.nl_ints = p->nl_ints;
   a.nkb = p->nkb;
   a.npw_beta = p->npw_max;
   fused_layout(p, precision, s, &a.nl_off, &a.loc_off);
@@ -1039,7 +1067,10 @@ int pwk_plan_create(pwk_plan** out, const double* A, int N1, int N2, int N3, int
   {
     unsigned* hm = reinterpret_cast<unsigned*>(d_vsum + 1);
     TRY(launch_fx_field(p->N, 1, vloc_r, p->d_Vfx, hm, reinterpret_cast<int*>(hm + 1), 0));
-    TRYC(cudaMemcpy(&p->v_exp, hm + 1, sizeof(int), cudaMemcpyDeviceToHost), "cudaMemcpy(vexp)");
+    unsigned v[2] = {0u, 0u};   // the largest high word of V, its exponent
+    TRYC(cudaMemcpy(v, hm, sizeof(v), cudaMemcpyDeviceToHost), "cudaMemcpy(vexp)");
+    p->v_exp = (int)v[1];
+    TRY(choose_projector_sums(p, v[0]));
   }
   TRYC(cudaMemset(d_vsum, 0, sizeof(double)), "cudaMemset");
   sum_kernel<<<1, 256>>>((size_t)p->Nr, vloc_r, d_vsum); note_launch();

@@ -99,6 +99,7 @@ struct pwk_plan {
   float* d_V32 = nullptr;         // transposed [l2][l3][l1]
   int2* d_Vfx = nullptr;          // transposed [l2][l3][l1], limb pairs of V 2^(63 - v_exp)
   int v_exp = 0;
+  bool nl_ints = false;           // FP64 projector sums of H as integers (nl_fused.cuh): V large enough
   double v_mean = 0.0;           // average of V over the grid (diagonal of the local term)
   pwk::SphereMap self;
   // window-specialised kernel tables (|m_i| <= (N-1)/4 on every sphere of the plan)
@@ -164,6 +165,7 @@ struct FusedArgs {
   // nonlocal projector terms fused into the kernel (nl_fused.cuh); beta == null: none
   const void* beta = nullptr;      // [nk][nkb][npw_beta] complex of the arithmetic type
   const int* bexp = nullptr;       // FP64: [nk][nkb] exponents of the projectors
+  bool nl_ints = false;            // FP64: the plan's choice of the integer sums for H alone
   const void* Dm = nullptr;        // [nkb][nkb] real of the arithmetic type
   const void* qm = nullptr;        // [nkb][nkb] or null (S = 1)
   void* sout = nullptr;            // S C output (io type) or null

@@ -250,6 +250,30 @@ def test_projector_terms_in_limbs(N, nat, lset, kind, spread):
 
 
 @pytest.mark.parametrize("path,kind", [(2, 1), (3, 0), (3, 1), (3, 2)])
+@pytest.mark.parametrize("field,strength", [(0.0, 1.0), (1e-6, 1.0), (1.0, 1e4)])
+def test_h_in_every_component_where_the_projectors_lead(path, kind, field, strength):
+    """H C of vectors that fall off like the projectors, V = 0 or weak beside them: every
+    component to the rounding of sums in doubles and of the local term.  Bound: that of S below,
+    with the kinetic term (its table to four roundings), and 1e-15 max |V| |C| for the local one."""
+    N, lset = 24, (0, 1)
+    base = problem(N, lset=lset)
+    prob = problem(N, V_r=field * base.V_r, lset=lset)
+    prob.beta = strength * prob.beta
+    r = np.random.default_rng(7)
+    n = int(prob.npw[0])
+    g = prob.kpts[0][None, :] + prob.miller[0][:n] @ prob.B
+    t = np.sum(g * g, axis=1)
+    x = np.zeros((1, 4, prob.npw_max), complex)
+    x[0, :, :n] = np.exp(-t / 3) * (r.standard_normal((4, n)) + 1j * r.standard_normal((4, n)))
+    y = apply(prob, x, (kind, 128, 1), path=path)[0, :, :n]
+    b, v = np.abs(prob.beta[0][:, :n]), np.abs(x[0, :, :n])
+    moduli = ((v @ b.T) @ np.abs(prob.D)) @ b
+    bound = 2.0 ** -53 * 2 * ((n / 32 + 5 + 2 * prob.nkb + 4) * moduli + 4 * t * v)
+    bound += 1e-15 * np.max(np.abs(prob.V_r)) * np.linalg.norm(v, axis=1)[:, None]
+    assert np.all(np.abs(y - reference(prob, 0, x[0])) <= bound)
+
+
+@pytest.mark.parametrize("path,kind", [(2, 1), (3, 0), (3, 1), (3, 2)])
 def test_s_in_every_component(path, kind):
     """S C of vectors that fall off like the projectors (smallest components 1e-6 of the largest):
     every component to the rounding of sums in doubles, whatever its size.  Bound: u times the
