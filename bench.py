@@ -85,8 +85,8 @@ TRAFFIC = {
     "rr_kernel": {"bytes": 8 * (10562816 + 44288), "profile": "profiles/rr_kernel_davidson_fcc64k_20b.md",
                   "sources": ["rr.cu", "solvers.h"], "digest": "561669374c49"},
     "fused_window_kernel<float,float,24,6>": {
-        "bytes": 48416683 + 4098645, "profile": "profiles/hpsi_step_kernels_fcc512k_20b_fp32.md",
-        "sources": ["fused_window.cuh", "fft_line.cuh", "hpsi_f32.cu"], "digest": "573ad38aa930"},
+        "bytes": 48409941 + 4088405, "profile": "profiles/hpsi_step_kernels_fcc512k_20b_fp32.md",
+        "sources": ["fused_window.cuh", "fft_line.cuh", "hpsi_f32.cu"], "digest": "dbb74c7b7ac9"},
     "nl_project_kernel<float,float,9>": {
         "bytes": 65060011 + 12288, "profile": "profiles/hpsi_step_kernels_fcc512k_20b_fp32.md",
         "sources": ["nonlocal.cu"], "digest": "67c9475f7eb9"},
@@ -94,9 +94,9 @@ TRAFFIC = {
         "bytes": 66527147 + 159061, "profile": "profiles/hpsi_step_kernels_fcc512k_20b_fp32.md",
         "sources": ["nonlocal.cu"], "digest": "67c9475f7eb9"},
     "fused_window_kernel_nl<float,float,24,6>": {
-        "bytes": 68634965 + 11855189, "profile": "profiles/fused_window_kernel_nl_hpsi_fcc512k_20b_fp32.md",
+        "bytes": 68629077 + 11927797, "profile": "profiles/fused_window_kernel_nl_hpsi_fcc512k_20b_fp32.md",
         "sources": ["fused_window.cuh", "fft_line.cuh", "nl_fused.cuh", "hpsi_f32_nl.cu"],
-        "digest": "c7071c70bae3"},
+        "digest": "bdf361b8ae02"},
 }
 
 

@@ -160,10 +160,11 @@ int pwk_supported_grid(int N);
  *              must not otherwise overlap it
  * PWK_FP64: the 2-norm of the error of a band is that of FP64 transforms, about 2e-16 of the
  * band's result (5e-16 at most in the tests).  The transforms, and with path 3 the projector sums
- * of a call for H alone, run in 64-bit integers scaled by the vector, V(r) and the projectors as
- * a whole: like a transform in FP64 they spread their rounding over all components alike, so a
- * component far below the others is exact to the rounding of the largest, not of itself (S psi of
- * pwk_hspsi_batched is exact to rounding in every component).  A vector with a component that is
+ * of a call for H alone where max |V| is no smaller than the projector matrix, run in 64-bit integers
+ * scaled by the vector, V(r) and the projectors as a whole: like a transform in FP64 the local term
+ * spreads its rounding over all components alike, so a component far below the others is exact to
+ * the rounding of the largest, not of itself (S psi of pwk_hspsi_batched is exact to rounding in
+ * every component, and so is H psi with V = 0).  A vector with a component that is
  * not finite gives NaN in all its components.
  * One launch on `stream` with path 3, else three (projections, local and kinetic terms, nonlocal
  * add-back); the
